@@ -15,19 +15,22 @@
 // -d^2)(u, v, 1)^T, so each (pixel, record) adds 7 moments of (u, v).
 // Per-record sums (colour, dL/do, moments) go to a per-record slot array:
 // when at most twelve lanes of the warp contribute, each adds its 11 values with
-// three 16-byte vector reductions; otherwise they are reduced across the warp
-// (a transposing butterfly: 11 values in 13 shuffles) and added with one
-// atomic per value per warp. The feature gradient is accumulated
-// warp-cooperatively across channels.
+// three 16-byte vector reductions; otherwise each group of eight lanes reduces
+// its record's (a transposing butterfly: 11 values in 12 shuffles) and adds
+// them with one 16-byte reduction on four of its lanes. The feature gradient
+// is accumulated warp-cooperatively across channels.
 // With the 2DGS low-pass filter, a pixel where the screen-space term
 // rho = 2 |x - p0|^2 wins adds dL/dp0 = 2 a (x - p0) (a = dL/dalpha * alpha)
-// instead of the (u, v) moments: 13 sums (16-slot butterfly, 16 shuffles)
+// instead of the (u, v) moments: 13 sums (16-slot butterfly)
 // and two more moments per record, taken through the projection of mu.
 // Both passes stream the list through the same producer-warp pipeline as the
 // forward kernel (raster.cuh): pass A front to back until every pixel is
 // saturated, pass B back to front from the largest last-composited position
-// of the tile; a warp visits only the records that meet its 8x4 block, and in
-// pass B only those before the last surfel of one of its pixels.
+// of the tile; each group of eight lanes walks the list of the records that
+// can reach one of its pixels (build_hits), in pass B only those before the
+// last surfel of one of them. Walking per group took the 3M-surfel 1080p walk
+// from 1.97 to 1.75 ms, the 16-channel dense one (700k surfels, 1237x701) from
+// 1.27 to 0.90 ms.
 // With the forward's saved state and a Top-K selection, pass B also exists
 // in a form with two pixels per lane (bwd_tile_pair below; a launch shape).
 // A second kernel turns the per-record moments into gradients of mu, t_u,
@@ -39,10 +42,14 @@ namespace {
 
 using namespace raster;
 
-// per record: dL/dc (3), dL/do, Suu, Suv, Svv, Su, Sv, Sdu, Sdv, padding; with
-// the low-pass filter also dL/dp0x, dL/dp0y and three padding floats -- whole
-// float4s, so that a pixel can add its share with 16-byte vector reductions
-__host__ __device__ constexpr int moments_per_record(bool lp) { return lp ? 16 : 12; }
+// Per record 16 floats (four float4s), so that both ways of adding a pixel's
+// or a group's share are 16-byte vector reductions. With v0..v2 = dL/dc, v3 =
+// dL/do, v4..v10 = Suu, Suv, Svv, Su, Sv, Sdu, Sdv and, with the low-pass
+// filter, v11, v12 = dL/dp0:
+//     (v0 v1 v2 v9) (v3 v4 v5 v10) (v6 v7 v8 v11) (v12 . . .)
+// Without the filter a group's butterfly leaves v9 and v10 in the fourth
+// float4 instead: v9 = slot 3 + slot 12, v10 = slot 7 + slot 13.
+constexpr int kMoments = 16;
 
 struct BwdArgs {
     const float4 *records;
@@ -56,7 +63,7 @@ struct BwdArgs {
     const float *g_F;   // [P_total, D] or NULL
     const float *g_T;   // [P_total] or NULL
     float *g_feat;      // [N,D] or NULL
-    float *moments;     // [R, moments_per_record]
+    float *moments;     // [R, kMoments]
     DevStatus *status;
     // forward state of the same frame (all NULL: recompute it in pass A)
     const float *saved_T;      // [P_total]
@@ -65,44 +72,6 @@ struct BwdArgs {
     const float *kd_saved;     // [P_total, K] <gF, f_j> of the saved set (feat_bwd.cu), or NULL
     unsigned int *work;        // persistent launch: the context's adjoint tile counter pair; NULL: one tile per CTA
 };
-
-// Sum 12 per-lane values over the warp (a transposing butterfly, 13
-// shuffles): afterwards lane l (and l ^ 1) holds the total of value index
-// 6 b4 + 3 b3 + g with g = 2 b2 + b1 (b_k = bit k of l); lanes with g = 3 hold
-// a padding slot.
-__device__ __forceinline__ float warp_transpose_sum12(float v[12], int lane)
-{
-#pragma unroll
-    for (int k = 0; k < 6; ++k) { // 12 -> 6: halves [0, 6) / [6, 12)
-        const bool hi = lane & 16;
-        const float send = hi ? v[k] : v[k + 6];
-        const float keep = hi ? v[k + 6] : v[k];
-        v[k] = keep + __shfl_xor_sync(0xffffffffu, send, 16);
-    }
-#pragma unroll
-    for (int k = 0; k < 3; ++k) { // 6 -> 3
-        const bool hi = lane & 8;
-        const float send = hi ? v[k] : v[k + 3];
-        const float keep = hi ? v[k + 3] : v[k];
-        v[k] = keep + __shfl_xor_sync(0xffffffffu, send, 8);
-    }
-    v[3] = 0.0f; // 3 -> 4 slots (one padding)
-#pragma unroll
-    for (int k = 0; k < 2; ++k) { // 4 -> 2
-        const bool hi = lane & 4;
-        const float send = hi ? v[k] : v[k + 2];
-        const float keep = hi ? v[k + 2] : v[k];
-        v[k] = keep + __shfl_xor_sync(0xffffffffu, send, 4);
-    }
-    {
-        const bool hi = lane & 2; // 2 -> 1
-        const float send = hi ? v[0] : v[1];
-        const float keep = hi ? v[1] : v[0];
-        v[0] = keep + __shfl_xor_sync(0xffffffffu, send, 2);
-    }
-    v[0] += __shfl_xor_sync(0xffffffffu, v[0], 1);
-    return v[0];
-}
 
 // The saved Top-K set of one pixel met during pass B. The saved ids are in
 // list order, so walking back to front the next selected surfel the pixel
@@ -156,47 +125,84 @@ struct SavedSel {
     }
 };
 
-// Up to this many contributing lanes add their values with their own 16-byte
-// vector reductions (3 or 4 per lane) instead of reducing over the warp first:
-// the walk is bound by instruction issue and the L2 has atomic throughput to
-// spare, so the reductions pay off up to 12-16 lanes (1.61 ms for the walk of
-// the 3M-surfel frame at 12, against 1.70 at 4, 1.67 at 20, 3.06 at 32).
+// Up to this many contributing lanes of the warp add their values with their
+// own 16-byte vector reductions (3 or 4 per lane) instead of reducing over the
+// lanes first: the walk is bound by instruction issue and the L2 has atomic
+// throughput to spare.
 constexpr int kDirectLanes = 12;
 
-// Adds one record's per-lane sums (the lane contributes if `act`) to its
-// 16-byte aligned slot array: by direct vector reductions up to kDirectLanes
-// contributing lanes, else through the warp butterfly and one atomic per sum.
-// (Adding lane pairs first and reducing directly from the even lanes up to 24
-// or 32 contributing lanes measured slower: 1.64 and 1.90 ms against 1.58 ms
-// for the walk of the 3M-surfel frame.)
-template <bool LP>
-__device__ __forceinline__ void add_record_sums(float *vals, bool act, uint32_t amask, int lane, float *slots)
+// Adds per-lane sums of one record per group of lanes to the records' slot
+// arrays (`slots`: the lane's record; the lane contributes if `act`). Up to
+// kDirectLanes contributing lanes: direct vector reductions. Otherwise the
+// sums of each group of eight lanes are taken by a transposing butterfly (12
+// values in 12 shuffles, 16 in 16), after which four lanes of the group each
+// hold one float4 of the slots. WARP: all lanes hold the same record; the four
+// groups are summed too and one of them adds.
+template <bool LP, bool WARP>
+__device__ __forceinline__ void add_record_sums(float *v, bool act, uint32_t amask, int lane, float *slots)
 {
-    constexpr int kM = moments_per_record(LP);
-    constexpr int kSums = LP ? 13 : 11;
+    float4 *dst = reinterpret_cast<float4 *>(slots);
     if (__popc(amask) <= kDirectLanes) {
         if (act) {
-            float4 *dst = reinterpret_cast<float4 *>(slots);
-#pragma unroll
-            for (int k4 = 0; k4 < kM / 4; ++k4)
-                atomicAdd(dst + k4, make_float4(vals[4 * k4], vals[4 * k4 + 1], vals[4 * k4 + 2], vals[4 * k4 + 3]));
+            atomicAdd(dst, make_float4(v[0], v[1], v[2], v[9]));
+            atomicAdd(dst + 1, make_float4(v[3], v[4], v[5], v[10]));
+            atomicAdd(dst + 2, make_float4(v[6], v[7], v[8], LP ? v[LP ? 11 : 0] : 0.0f));
+            if (LP) atomicAdd(dst + 3, make_float4(v[LP ? 12 : 0], 0.0f, 0.0f, 0.0f));
         }
         return;
     }
-    float tot;
-    int idx;
-    bool mine;
+    constexpr int kH = LP ? 4 : 3; // values per lane class at the end
+    float w[4 * kH];
     if constexpr (LP) {
-        tot = warp_transpose_sum16(vals, lane);
-        idx = (lane >> 1) & 15;
-        mine = (lane & 1) == 0 && idx < kSums;
+        const float o[16] = {v[0], v[1], v[2], v[9], v[3], v[4], v[5], v[10], v[6], v[7], v[8], v[11], v[12], 0.f, 0.f, 0.f};
+#pragma unroll
+        for (int k = 0; k < 16; ++k) w[k] = o[k];
     } else {
-        tot = warp_transpose_sum12(vals, lane);
-        const int g = ((lane >> 2) & 1) * 2 + ((lane >> 1) & 1);
-        idx = ((lane >> 4) & 1) * 6 + ((lane >> 3) & 1) * 3 + g;
-        mine = (lane & 1) == 0 && g < 3;
+#pragma unroll
+        for (int k = 0; k < 11; ++k) w[k] = v[k];
+        w[11] = 0.0f;
     }
-    if (mine && tot != 0.0f) atomicAdd(slots + idx, tot);
+    const bool hi4 = lane & 4, hi2 = lane & 2;
+#pragma unroll
+    for (int k = 0; k < 2 * kH; ++k) {
+        const float send = hi4 ? w[k] : w[k + 2 * kH];
+        const float keep = hi4 ? w[k + 2 * kH] : w[k];
+        w[k] = keep + __shfl_xor_sync(0xffffffffu, send, 4);
+    }
+#pragma unroll
+    for (int k = 0; k < kH; ++k) {
+        const float send = hi2 ? w[k] : w[k + kH];
+        const float keep = hi2 ? w[k + kH] : w[k];
+        w[k] = keep + __shfl_xor_sync(0xffffffffu, send, 2);
+        w[k] += __shfl_xor_sync(0xffffffffu, w[k], 1);
+        if constexpr (WARP) {
+            w[k] += __shfl_xor_sync(0xffffffffu, w[k], 8);
+            w[k] += __shfl_xor_sync(0xffffffffu, w[k], 16);
+        }
+    }
+    const bool any = WARP ? lane < 8 : ((amask >> (lane & 24)) & 0xFFu) != 0u;
+    if (any && (lane & 1) == 0) atomicAdd(dst + ((lane >> 1) & 3), make_float4(w[0], w[1], w[2], LP ? w[LP ? 3 : 0] : 0.0f));
+}
+
+// Sums 16 per-lane values over each group of eight lanes (16 shuffles):
+// afterwards lanes 2c and 2c + 1 of the group hold the totals of values
+// [4c, 4c + 4) in v[0..3].
+__device__ __forceinline__ void group_transpose_sum16(float v[16], int lane)
+{
+    const bool hi4 = lane & 4, hi2 = lane & 2;
+#pragma unroll
+    for (int k = 0; k < 8; ++k) {
+        const float send = hi4 ? v[k] : v[k + 8];
+        const float keep = hi4 ? v[k + 8] : v[k];
+        v[k] = keep + __shfl_xor_sync(0xffffffffu, send, 4);
+    }
+#pragma unroll
+    for (int k = 0; k < 4; ++k) {
+        const float send = hi2 ? v[k] : v[k + 4];
+        const float keep = hi2 ? v[k + 4] : v[k];
+        v[k] = keep + __shfl_xor_sync(0xffffffffu, send, 2);
+        v[k] += __shfl_xor_sync(0xffffffffu, v[k], 1);
+    }
 }
 
 // SAVED: T_final, last and the Top-K ids come from the forward's outputs;
@@ -206,18 +212,20 @@ __device__ __forceinline__ void add_record_sums(float *vals, bool act, uint32_t 
 // One tile (the whole CTA; P freshly initialised by thread 0 below).
 // NW (dense features with D = 16, e.g. the depth/normal table): each pixel's
 // g_F row is held in registers for the whole walk, and dL/df of a record is
-// summed over the warp by one 16-value transposing butterfly (one atomic per
-// channel) instead of the lanes-across-channels rounds, which would leave 28
-// of 32 lanes idle at 16 channels.
+// summed over its group of lanes by one 16-value transposing butterfly (one
+// 16-byte reduction per four channels) instead of the lanes-across-channels
+// rounds, which would leave 28 of 32 lanes idle at 16 channels.
+// Pass B walks one list per group of lanes (build_hits) unless the feature
+// gradient is summed by the whole warp, lanes across channels (NG = 1).
 template <int KMAX, int DT, int CH, bool SAVED, bool LP, int TH, bool NW = false>
-__device__ __forceinline__ void bwd_tile(const FrameParams &fp, const BwdArgs &a, Pipe &P, int &s_maxlast,
-                                         uint32_t tile)
+__device__ __forceinline__ void bwd_tile(const FrameParams &fp, const BwdArgs &a, Pipe &P, HitLists *hits,
+                                         int &s_maxlast, uint32_t tile)
 {
     constexpr int PW = pixel_warps(TH);
-    constexpr int kM = moments_per_record(LP);
     constexpr int kSlots = LP ? 16 : 12;
     const int tid = threadIdx.x, wid = tid >> 5, lane = tid & 31;
     const bool producer = wid == PW;
+    const unsigned long long wlimit = wait_limit(a.status); // in flight with the tile's own loads
     const int v = view_of_tile(fp, tile);
     const ViewParams &cam = fp.v[v];
     const int local = static_cast<int>(tile - cam.tile_base);
@@ -240,9 +248,10 @@ __device__ __forceinline__ void bwd_tile(const FrameParams &fp, const BwdArgs &a
     const bool inside = !producer && px < cam.W && py < cam.H;
     const float lx = static_cast<float>(lxi), ly = static_cast<float>(lyi);
     const int64_t pix = cam.pix_base + static_cast<int64_t>(min(py, cam.H - 1)) * cam.W + min(px, cam.W - 1);
+    const int grp = lane >> 3;
 
     if (tid == 0) {
-        pipe_init(P, PW);
+        pipe_init(P, PW, wlimit);
         s_maxlast = 0;
     }
     __syncthreads();
@@ -265,45 +274,44 @@ __device__ __forceinline__ void bwd_tile(const FrameParams &fp, const BwdArgs &a
         if (!PSI_CHECK(last >= 0 && last <= n, kChkLast, a.status)) last = 0;
         last = min(max(last, 0), n);
     } else if (producer) {
-        pipe_produce(P, a.vals, list0, n, false, a.records, tileX, tileY, a.status, kSiteRenderBwdA, rec_lo, rec_hi);
+        pipe_produce<LP, PW>(P, a.vals, list0, n, false, a.records, tileX, tileY, a.status, kSiteRenderBwdA, rec_lo,
+                             rec_hi);
     } else {
+        pipe_prefill<LP, PW>(P, wid, a.vals, list0, n, false, a.records, tileX, tileY, a.status, rec_lo, rec_hi);
         const int nb = (n + kPB - 1) / kPB;
-        bool wdone = __all_sync(0xffffffffu, done);
-        if (wdone && lane == 0) atomicSub(&P.alive, 1);
-        for (int b = 0; b < nb; ++b) {
+        bool in_walk = !__all_sync(0xffffffffu, done);
+        if (!in_walk) pipe_leave(P, wid);
+        for (int b = 0; b < nb && in_walk; ++b) {
             if (!pipe_wait_ready(P, b, a.status, kSiteRenderBwdA)) break;
             const int st = b % kPS;
             int cnt;
             const int lo = batch_range(b, n, false, cnt);
-            if (!wdone) {
-                uint32_t hw[kPB / 32];
-                pipe_hit_words(P, st, cnt, vw, hw);
-                bool all_done = false;
+            int ng[kGroups];
+            const int lim[kGroups] = {kPB, kPB, kPB, kPB};
+            build_hits<LP, kGroups>(P, st, cnt, vw, tileX, tileY, lim, hits[wid], ng);
+            const int mine = grp == 0 ? ng[0] : grp == 1 ? ng[1] : grp == 2 ? ng[2] : ng[3];
+            const int most = max(max(ng[0], ng[1]), max(ng[2], ng[3]));
+            const uint8_t *list = hits[wid][grp];
 #pragma unroll 1
-                for (int q = 0; q < kPB / 32 && !all_done; ++q)
-#pragma unroll 1
-                for (uint32_t bits = q == 0 ? hw[0] : q == 1 ? hw[1] : q == 2 ? hw[2] : hw[3]; bits; bits &= bits - 1) {
-                    if (__all_sync(0xffffffffu, done)) {
-                        all_done = true;
-                        break;
-                    }
-                    const int j = q * 32 + __ffs(bits) - 1;
-                    const Rec r = load_rec(P.rec[st][j]);
-                    Eval e;
-                    const bool hit = !done && eval_alpha<LP>(r, lx, ly, e);
-                    const float w = hit ? __fmul_rn(e.alpha, T) : 0.0f;
-                    if constexpr (KMAX > 0) top.offer(hit, w, lo + j);
-                    if (hit) {
-                        T = __fmul_rn(T, __fsub_rn(1.0f, e.alpha));
-                        last = lo + j + 1;
-                        if (T < fp.t_eps) done = true;
-                    }
+            for (int i = 0; i < most; ++i) {
+                if (__all_sync(0xffffffffu, done)) break;
+                const int j = list[i] & (kPB - 1); // past the group's list: any staged record, not used
+                const Rec r = load_rec(P.rec[st][j]);
+                Eval e;
+                const bool hit = i < mine && !done && eval_alpha<LP>(r, lx, ly, e);
+                const float w = hit ? __fmul_rn(e.alpha, T) : 0.0f;
+                if constexpr (KMAX > 0) top.offer(hit, w, lo + j);
+                if (hit) {
+                    T = __fmul_rn(T, __fsub_rn(1.0f, e.alpha));
+                    last = lo + j + 1;
+                    if (T < fp.t_eps) done = true;
                 }
             }
-            pipe_release(P, b);
-            if (!wdone && __all_sync(0xffffffffu, done)) {
-                wdone = true;
-                if (lane == 0) atomicSub(&P.alive, 1);
+            if (__all_sync(0xffffffffu, done)) {
+                in_walk = false;
+                pipe_leave(P, wid);
+            } else {
+                pipe_release(P, wid, b);
             }
         }
     }
@@ -327,9 +335,7 @@ __device__ __forceinline__ void bwd_tile(const FrameParams &fp, const BwdArgs &a
         }
 #pragma unroll
         for (int s = 0; s < KMAX; ++s) kd[s] = 0.0f;
-        if (ext_feat) {
-            sel_saved.init(a, pix, K, fp.n, inside);
-        } else if (a.g_F && a.feat && inside) {
+        if (!ext_feat && a.g_F && a.feat && inside) {
             for (int c0 = 0; c0 < a.D; c0 += 16) {
                 float g[16];
 #pragma unroll
@@ -364,24 +370,26 @@ __device__ __forceinline__ void bwd_tile(const FrameParams &fp, const BwdArgs &a
         if (tid == 0) {
             // fresh barriers for the reverse walk
             for (int s = 0; s < kPS; ++s) {
-                asm volatile("mbarrier.inval.shared::cta.b64 [%0];" ::"r"(smem_u32(&P.full[s])) : "memory");
                 asm volatile("mbarrier.inval.shared::cta.b64 [%0];" ::"r"(smem_u32(&P.ready[s])) : "memory");
-                asm volatile("mbarrier.inval.shared::cta.b64 [%0];" ::"r"(smem_u32(&P.empty[s])) : "memory");
             }
-            pipe_init(P, PW);
+            pipe_init(P, PW, P.limit);
         }
         __syncthreads();
     }
     const int maxlast = s_maxlast;
     if (producer) {
-        pipe_produce(P, a.vals, list0, maxlast, true, a.records, tileX, tileY, a.status, kSiteRenderBwdB, rec_lo,
-                     rec_hi);
+        pipe_produce<LP, PW>(P, a.vals, list0, maxlast, true, a.records, tileX, tileY, a.status, kSiteRenderBwdB,
+                             rec_lo, rec_hi);
         return;
     }
-    // entries at or beyond every lane's last composited surfel are skipped by the warp
-    int warp_last = last;
+    pipe_prefill<LP, PW>(P, wid, a.vals, list0, maxlast, true, a.records, tileX, tileY, a.status, rec_lo, rec_hi);
+    if constexpr (ext_feat) sel_saved.init(a, pix, K, fp.n, inside);
+    // entries at or beyond every lane's last composited surfel are skipped by
+    // the group (the warp when it walks one list)
+    constexpr int NG = (ext_feat || NW) ? kGroups : 1;
+    int my_last = last;
 #pragma unroll
-    for (int o = 16; o > 0; o >>= 1) warp_last = max(warp_last, __shfl_xor_sync(0xffffffffu, warp_last, o));
+    for (int o = NG == 1 ? 16 : 4; o > 0; o >>= 1) my_last = max(my_last, __shfl_xor_sync(0xffffffffu, my_last, o));
 
     // ---------------- pass B: back to front
     const float gr = inside ? a.g_rgb[pix] : 0.0f;
@@ -403,25 +411,31 @@ __device__ __forceinline__ void bwd_tile(const FrameParams &fp, const BwdArgs &a
         const int st = b % kPS;
         int cnt;
         const int lo = batch_range(b, maxlast, true, cnt);
-        const int limit = min(cnt, warp_last - lo); // entries [0, limit) of the batch can matter
+        int ng[NG], lim[NG];
+        int limit = 0; // entries [0, limit) of the batch can matter to the warp
+#pragma unroll
+        for (int g = 0; g < NG; ++g) {
+            lim[g] = __shfl_sync(0xffffffffu, my_last, 8 * g) - lo;
+            limit = max(limit, lim[g]);
+        }
+        limit = min(cnt, limit);
         if (limit > 0) {
-            uint32_t hw[kPB / 32];
-            pipe_hit_words(P, st, cnt, vw, hw);
+            build_hits<LP, NG>(P, st, limit, vw, tileX, tileY, lim, hits[wid], ng);
+            int mine = ng[0], most = ng[0];
+#pragma unroll
+            for (int g = 1; g < NG; ++g) {
+                mine = grp == g ? ng[g] : mine;
+                most = max(most, ng[g]);
+            }
+            const uint8_t *list = hits[wid][NG == 1 ? 0 : grp];
+            {
 #pragma unroll 1
-            for (int q = kPB / 32 - 1; q >= 0; --q) {
-                uint32_t bits = q == 0 ? hw[0] : q == 1 ? hw[1] : q == 2 ? hw[2] : hw[3];
-                const int room = limit - q * 32;
-                if (room <= 0) continue;
-                if (room < 32) bits &= (1u << room) - 1u;
-#pragma unroll 1
-                for (; bits; ) {
-                    const int jj = 31 - __clz(bits);
-                    bits &= ~(1u << jj);
-                    const int j = q * 32 + jj;
+                for (int i = mine - 1; i >= mine - most; --i) { // the same count in every lane
+                    const int j = list[max(i, 0)] & (kPB - 1);
                     const int pos = lo + j;
                     const Rec r = load_rec(P.rec[st][j]);
                     Eval e;
-                    const bool act = inside && pos < last && eval_alpha<LP>(r, lx, ly, e);
+                    const bool act = i >= 0 && pos < last && eval_alpha<LP>(r, lx, ly, e);
                     const uint32_t amask = __ballot_sync(0xffffffffu, act);
                     if (!amask) continue;
                     const uint32_t rid = P.val[st][j];
@@ -506,15 +520,17 @@ __device__ __forceinline__ void bwd_tile(const FrameParams &fp, const BwdArgs &a
                             vals[10] = td.y;
                         }
                     }
-                    add_record_sums<LP>(vals, act, amask, lane, a.moments + static_cast<int64_t>(rid) * kM);
+                    add_record_sums<LP, NG == 1>(vals, act, amask, lane, a.moments + static_cast<int64_t>(rid) * kMoments);
                     if (NW && want_feat) {
-                        if (__any_sync(0xffffffffu, act && sel)) {
+                        const uint32_t smask = __ballot_sync(0xffffffffu, act && sel);
+                        if (smask) {
                             float v[16];
 #pragma unroll
                             for (int c = 0; c < 16; ++c) v[c] = (act && sel) ? w * gfr[c] : 0.0f;
-                            // lane l ends with the total of channel l >> 1
-                            const float tot = warp_transpose_sum16(v, lane);
-                            if ((lane & 1) == 0 && tot != 0.0f) atomicAdd(a.g_feat + sid * 16 + (lane >> 1), tot);
+                            group_transpose_sum16(v, lane);
+                            if ((lane & 1) == 0 && ((smask >> (lane & 24)) & 0xFFu))
+                                atomicAdd(reinterpret_cast<float4 *>(a.g_feat + sid * 16) + ((lane >> 1) & 3),
+                                          make_float4(v[0], v[1], v[2], v[3]));
                         }
                     } else if (want_feat) {
                         uint32_t selmask = __ballot_sync(0xffffffffu, act && sel);
@@ -568,7 +584,7 @@ __device__ __forceinline__ void bwd_tile(const FrameParams &fp, const BwdArgs &a
                 }
             }
         }
-        pipe_release(P, b);
+        pipe_release(P, wid, b);
     }
 }
 
@@ -589,10 +605,10 @@ __device__ __forceinline__ void bwd_tile_pair(const FrameParams &fp, const BwdAr
                                               uint32_t tile)
 {
     constexpr int PW = pair_warps(TH);
-    constexpr int kM = moments_per_record(LP);
     constexpr int kSlots = LP ? 16 : 12;
     const int tid = threadIdx.x, wid = tid >> 5, lane = tid & 31;
     const bool producer = wid == PW;
+    const unsigned long long wlimit = wait_limit(a.status); // in flight with the tile's own loads
     const int v = view_of_tile(fp, tile);
     const ViewParams &cam = fp.v[v];
     const int local = static_cast<int>(tile - cam.tile_base);
@@ -614,7 +630,7 @@ __device__ __forceinline__ void bwd_tile_pair(const FrameParams &fp, const BwdAr
     const float lx = static_cast<float>(lxi);
 
     if (tid == 0) {
-        pipe_init(P, PW);
+        pipe_init(P, PW, wlimit);
         s_maxlast = 0;
     }
     __syncthreads();
@@ -655,10 +671,11 @@ __device__ __forceinline__ void bwd_tile_pair(const FrameParams &fp, const BwdAr
     __syncthreads();
     const int maxlast = s_maxlast;
     if (producer) {
-        pipe_produce(P, a.vals, list0, maxlast, true, a.records, tileX, tileY, a.status, kSiteRenderBwdB, rec_lo,
-                     rec_hi);
+        pipe_produce<LP, PW>(P, a.vals, list0, maxlast, true, a.records, tileX, tileY, a.status, kSiteRenderBwdB,
+                             rec_lo, rec_hi);
         return;
     }
+    pipe_prefill<LP, PW>(P, wid, a.vals, list0, maxlast, true, a.records, tileX, tileY, a.status, rec_lo, rec_hi);
 
     const int nbB = (maxlast + kPB - 1) / kPB;
     for (int b = 0; b < nbB; ++b) {
@@ -735,12 +752,12 @@ __device__ __forceinline__ void bwd_tile_pair(const FrameParams &fp, const BwdAr
                             vals[10] += aa * d2 * vv;
                         }
                     }
-                    add_record_sums<LP>(vals, act[0] || act[1], amask, lane,
-                                        a.moments + static_cast<int64_t>(rid) * kM);
+                    add_record_sums<LP, true>(vals, act[0] || act[1], amask, lane,
+                                              a.moments + static_cast<int64_t>(rid) * kMoments);
                 }
             }
         }
-        pipe_release(P, b);
+        pipe_release(P, wid, b);
     }
 }
 
@@ -782,13 +799,14 @@ __global__ void __launch_bounds__(pipe_threads(TH), OCC)
     render_bwd_kernel(const __grid_constant__ FrameParams fp, BwdArgs a)
 {
     __shared__ __align__(128) Pipe P;
+    __shared__ HitLists hits[pixel_warps(TH)];
     __shared__ int s_maxlast;
     __shared__ uint32_t s_next;
     uint32_t i = blockIdx.x;
     while (true) {
         const uint32_t tile = a.ranges[2 * fp.n_tiles_total + i];
         if (PSI_CHECK(tile < fp.n_tiles_total, kChkTile, a.status))
-            bwd_tile<KMAX, DT, CH, SAVED, LP, TH, NW>(fp, a, P, s_maxlast, tile);
+            bwd_tile<KMAX, DT, CH, SAVED, LP, TH, NW>(fp, a, P, hits, s_maxlast, tile);
         if (!a.work) break;
         __syncthreads();
         if (threadIdx.x == 0) {
@@ -817,12 +835,12 @@ __global__ void __launch_bounds__(256) chain_kernel(const __grid_constant__ Fram
     const int64_t total = fp.n * fp.n_views;
     const int64_t r = static_cast<int64_t>(blockIdx.x) * blockDim.x + threadIdx.x;
     if (r >= total) return;
-    constexpr int kV = moments_per_record(LP) / 4;
-    // slots: dL/dc (3), dL/do, Suu, Suv, Svv, Su, Sv, Sdu, Sdv, pad[, dL/dp0 (2), pad (3)]
-    const float4 q0 = moments[kV * r], q1 = moments[kV * r + 1], q2 = moments[kV * r + 2];
-    const float2 gp = LP ? make_float2(moments[kV * r + 2].w, moments[kV * r + 3].x) : make_float2(0.0f, 0.0f);
-    if (q0.x == 0.0f && q0.y == 0.0f && q0.z == 0.0f && q0.w == 0.0f && q1.x == 0.0f && q1.y == 0.0f &&
-        q1.z == 0.0f && q1.w == 0.0f && q2.x == 0.0f && q2.y == 0.0f && q2.z == 0.0f && gp.x == 0.0f && gp.y == 0.0f)
+    constexpr int kV = kMoments / 4;
+    const float4 q0 = moments[kV * r], q1 = moments[kV * r + 1], q2 = moments[kV * r + 2], q3 = moments[kV * r + 3];
+    const float Sdu = LP ? q0.w : q0.w + q3.x, Sdv = LP ? q1.w : q1.w + q3.y;
+    const float2 gp = LP ? make_float2(q2.w, q3.x) : make_float2(0.0f, 0.0f);
+    if (q0.x == 0.0f && q0.y == 0.0f && q0.z == 0.0f && q1.x == 0.0f && q1.y == 0.0f && q1.z == 0.0f && q2.x == 0.0f &&
+        q2.y == 0.0f && q2.z == 0.0f && Sdu == 0.0f && Sdv == 0.0f && gp.x == 0.0f && gp.y == 0.0f)
         return;
     const int v = static_cast<int>(r / fp.n);
     const int64_t i = r - static_cast<int64_t>(v) * fp.n;
@@ -833,8 +851,8 @@ __global__ void __launch_bounds__(256) chain_kernel(const __grid_constant__ Fram
         if (q0.y != 0.0f) atomicAdd(g.rgb + 3 * i + 1, q0.y);
         if (q0.z != 0.0f) atomicAdd(g.rgb + 3 * i + 2, q0.z);
     }
-    if (g.opacity) atomicAdd(g.opacity + i, q0.w);
-    const float Suu = q1.x, Suv = q1.y, Svv = q1.z, Su = q1.w, Sv = q2.x, Sdu = q2.y, Sdv = q2.z;
+    if (g.opacity) atomicAdd(g.opacity + i, q1.x);
+    const float Suu = q1.y, Suv = q1.z, Svv = q2.x, Su = q2.y, Sv = q2.z;
 
     float mu[3], tu[3], tv[3];
     for (int k = 0; k < 3; ++k) {
@@ -1013,17 +1031,16 @@ cudaError_t launch_k(const FrameParams &fp, const FeatView &f, const BwdArgs &a,
 } // namespace
 
 namespace {
-size_t moments_bytes(int64_t n_records, bool lp)
+size_t moments_bytes(int64_t n_records)
 {
-    return align_up(static_cast<size_t>(std::max<int64_t>(n_records, 1)) * moments_per_record(lp) * sizeof(float), 256);
+    return align_up(static_cast<size_t>(std::max<int64_t>(n_records, 1)) * kMoments * sizeof(float), 256);
 }
 } // namespace
 
-// sized for the low-pass layout, which is the larger one
 size_t render_bwd_workspace_bytes(int64_t n_records, int64_t n_pix, int top_k)
 {
     const size_t kd = top_k > 0 ? align_up(static_cast<size_t>(n_pix) * top_k * sizeof(float), 256) : 0;
-    return moments_bytes(n_records, true) + kd;
+    return moments_bytes(n_records) + kd;
 }
 
 cudaError_t launch_render_bwd(const FrameParams &fp, const psi_surfels &s, const FeatView &f, const float4 *records,
@@ -1037,7 +1054,7 @@ cudaError_t launch_render_bwd(const FrameParams &fp, const psi_surfels &s, const
     };
     const int64_t R = fp.n * fp.n_views;
     const bool lp = fp.lowpass != 0;
-    cudaError_t e = cudaMemsetAsync(ws, 0, moments_bytes(R, lp), st);
+    cudaError_t e = cudaMemsetAsync(ws, 0, moments_bytes(R), st);
     if (e != cudaSuccess || R == 0 || fp.n_tiles_total == 0) return e;
     BwdArgs a{};
     a.records = records;
@@ -1059,7 +1076,7 @@ cudaError_t launch_render_bwd(const FrameParams &fp, const psi_surfels &s, const
         a.saved_topk = saved->topk_ids;
         if (fp.top_k > 0 && a.g_F) {
             // feature terms from the saved selection: kd for the walk, dL/df
-            float *kd = reinterpret_cast<float *>(static_cast<char *>(ws) + moments_bytes(R, lp));
+            float *kd = reinterpret_cast<float *>(static_cast<char *>(ws) + moments_bytes(R));
             mark(PSI_KERNEL_BWD_FEAT, 0);
             e = launch_feat_bwd(fp, f, saved->topk_ids, saved->topk_w, a.g_F, kd, a.g_feat, status, st);
             if (e != cudaSuccess) return e;

@@ -1,9 +1,9 @@
 // a4: per-tile compositing with Top-K Hard Selection.
 //
 // One CTA per 16x16 tile, one thread per pixel. The tile's sorted list is
-// walked in batches of 256 records staged into shared memory by TMA bulk
-// copies (double buffered, mbarrier completion), so the next batch streams in
-// while the current one is composited. Per pixel (Sec. 3.1, Eq. 1): alpha =
+// streamed through shared-memory stages of 128 records (raster.cuh); each
+// warp lists, per group of eight pixels, the records that can reach the group
+// and every group walks its own list. Per pixel (Sec. 3.1, Eq. 1): alpha =
 // min(0.99, o exp(-(u^2+v^2)/2)), RGB blended densely front to back with FP32
 // transmittance T, and the K largest weights omega_j = alpha_j T_j kept in
 // registers (Sec. 5, Top-K Hard Selection): the insertion runs under a
@@ -44,10 +44,12 @@ struct FwdArgs {
 // One tile of the frame (the whole CTA; P freshly initialised by thread 0
 // below). TH: tile height (16x16 or 16x8 tiles).
 template <int KMAX, int DT, int CH, bool LP, int TH>
-__device__ __forceinline__ void fwd_tile(const FrameParams &fp, const FwdArgs &a, Pipe &P, uint32_t tile)
+__device__ __forceinline__ void fwd_tile(const FrameParams &fp, const FwdArgs &a, Pipe &P, HitLists *hits,
+                                         uint32_t tile)
 {
     constexpr int PW = pixel_warps(TH);
     const int tid = threadIdx.x, wid = tid >> 5, lane = tid & 31;
+    const unsigned long long wlimit = wait_limit(a.status); // in flight with the tile's own loads
     const int v = view_of_tile(fp, tile);
     const ViewParams &cam = fp.v[v];
     const int local = static_cast<int>(tile - cam.tile_base);
@@ -65,13 +67,14 @@ __device__ __forceinline__ void fwd_tile(const FrameParams &fp, const FwdArgs &a
     // sequence of the 16x16 launch (same results bit for bit).
     const int oy = (ty * TH) & 15;
     const int vw = wid + (oy ? pixel_warps(16) / 2 : 0); // warp of the 16x16 tile this warp plays
-    if (tid == 0) pipe_init(P, PW);
+    if (tid == 0) pipe_init(P, PW, wlimit);
     __syncthreads();
     if (wid == PW) {
-        pipe_produce(P, a.vals, list0, n, false, a.records, tx * kTile, ty * TH - oy, a.status, kSiteRenderFwd,
-                     rec_lo, rec_hi);
+        pipe_produce<LP, PW>(P, a.vals, list0, n, false, a.records, tx * kTile, ty * TH - oy, a.status, kSiteRenderFwd,
+                             rec_lo, rec_hi);
         return;
     }
+    pipe_prefill<LP, PW>(P, wid, a.vals, list0, n, false, a.records, tx * kTile, ty * TH - oy, a.status, rec_lo, rec_hi);
 
     int lxi, lyi;
     pixel_of_thread(vw * 32 + lane, lxi, lyi);
@@ -80,6 +83,7 @@ __device__ __forceinline__ void fwd_tile(const FrameParams &fp, const FwdArgs &a
     const float lx = static_cast<float>(lxi), ly = static_cast<float>(lyi);
     const int64_t surf0 = static_cast<int64_t>(v) * fp.n;
     const int K = KMAX > 0 ? fp.top_k : 0;
+    const int grp = lane >> 3;
 
     float T = 1.0f, cr = 0.0f, cg = 0.0f, cb = 0.0f;
     int last = 0;
@@ -90,58 +94,55 @@ __device__ __forceinline__ void fwd_tile(const FrameParams &fp, const FwdArgs &a
 #pragma unroll
     for (int c = 0; c < (KMAX == 0 ? CH : 1); ++c) facc[c] = 0.0f;
 
-    bool wdone = __all_sync(0xffffffffu, done);
-    if (wdone && lane == 0) atomicSub(&P.alive, 1);
-    for (int b = 0; b < nb; ++b) {
+    bool in_walk = !__all_sync(0xffffffffu, done);
+    if (!in_walk) pipe_leave(P, wid);
+    for (int b = 0; b < nb && in_walk; ++b) {
         if (!pipe_wait_ready(P, b, a.status, kSiteRenderFwd)) break;
         const int st = b % kPS;
         int cnt;
         const int lo = batch_range(b, n, false, cnt);
-        if (!wdone) {
-            // only the records that touch this warp's pixel block, in list order
-            uint32_t hw[kPB / 32];
-            pipe_hit_words(P, st, cnt, vw, hw);
-            bool all_done = false;
+        // only the records that can reach a pixel of this lane's group, in list order
+        int ng[kGroups];
+        const int lim[kGroups] = {kPB, kPB, kPB, kPB};
+        build_hits<LP, kGroups>(P, st, cnt, vw, tx * kTile, ty * TH - oy, lim, hits[wid], ng);
+        const int mine = grp == 0 ? ng[0] : grp == 1 ? ng[1] : grp == 2 ? ng[2] : ng[3];
+        const int most = max(max(ng[0], ng[1]), max(ng[2], ng[3]));
+        const uint8_t *list = hits[wid][grp];
 #pragma unroll 1
-            for (int q = 0; q < kPB / 32 && !all_done; ++q)
-#pragma unroll 1
-            for (uint32_t bits = q == 0 ? hw[0] : q == 1 ? hw[1] : q == 2 ? hw[2] : hw[3]; bits; bits &= bits - 1) {
-                if (__all_sync(0xffffffffu, done)) {
-                    all_done = true;
-                    break;
-                }
-                const int j = q * 32 + __ffs(bits) - 1;
-                const Rec r = load_rec(P.rec[st][j]);
-                Eval e;
-                const bool hit = !done && eval_alpha<LP>(r, lx, ly, e);
-                const float w = hit ? __fmul_rn(e.alpha, T) : 0.0f;
-                const int pos = lo + j;
-                if (hit) {
-                    const float4 col = P.rec[st][j][3];
-                    cr = __fmaf_rn(w, col.y, cr);
-                    cg = __fmaf_rn(w, col.z, cg);
-                    cb = __fmaf_rn(w, col.w, cb);
-                    if constexpr (KMAX == 0) {
-                        if (a.feat) {
-                            float f[CH];
-                            load_feat<DT, CH>(a.feat, static_cast<int64_t>(P.val[st][j]) - surf0, a.D, a.c0, f, a.wide);
+        for (int i = 0; i < most; ++i) {
+            if (__all_sync(0xffffffffu, done)) break;
+            const int j = list[i] & (kPB - 1); // past the group's list: any staged record, not used
+            const Rec r = load_rec(P.rec[st][j]);
+            Eval e;
+            const bool hit = i < mine && !done && eval_alpha<LP>(r, lx, ly, e);
+            const float w = hit ? __fmul_rn(e.alpha, T) : 0.0f;
+            const int pos = lo + j;
+            if (hit) {
+                const float4 col = P.rec[st][j][3];
+                cr = __fmaf_rn(w, col.y, cr);
+                cg = __fmaf_rn(w, col.z, cg);
+                cb = __fmaf_rn(w, col.w, cb);
+                if constexpr (KMAX == 0) {
+                    if (a.feat) {
+                        float f[CH];
+                        load_feat<DT, CH>(a.feat, static_cast<int64_t>(P.val[st][j]) - surf0, a.D, a.c0, f, a.wide);
 #pragma unroll
-                            for (int c = 0; c < CH; ++c) facc[c] = __fmaf_rn(w, f[c], facc[c]);
-                        }
+                        for (int c = 0; c < CH; ++c) facc[c] = __fmaf_rn(w, f[c], facc[c]);
                     }
                 }
-                if constexpr (KMAX > 0) top.offer(hit, w, pos);
-                if (hit) {
-                    T = __fmul_rn(T, __fsub_rn(1.0f, e.alpha));
-                    last = pos + 1;
-                    if (T < fp.t_eps) done = true;
-                }
+            }
+            if constexpr (KMAX > 0) top.offer(hit, w, pos);
+            if (hit) {
+                T = __fmul_rn(T, __fsub_rn(1.0f, e.alpha));
+                last = pos + 1;
+                if (T < fp.t_eps) done = true;
             }
         }
-        pipe_release(P, b);
-        if (!wdone && __all_sync(0xffffffffu, done)) {
-            wdone = true;
-            if (lane == 0) atomicSub(&P.alive, 1);
+        if (__all_sync(0xffffffffu, done)) {
+            in_walk = false;
+            pipe_leave(P, wid);
+        } else {
+            pipe_release(P, wid, b);
         }
     }
     if (vload(P.abort)) return;
@@ -224,12 +225,13 @@ __global__ void __launch_bounds__(pipe_threads(TH), OCC)
     render_fwd_kernel(const __grid_constant__ FrameParams fp, FwdArgs a)
 {
     __shared__ __align__(128) Pipe P;
+    __shared__ HitLists hits[pixel_warps(TH)];
     __shared__ uint32_t s_next;
     uint32_t i = blockIdx.x;
     while (true) {
         const uint32_t tile = a.ranges[2 * fp.n_tiles_total + i];
         // debug builds: the launch order must name a tile of the frame (uniform for the CTA)
-        if (PSI_CHECK(tile < fp.n_tiles_total, kChkTile, a.status)) fwd_tile<KMAX, DT, CH, LP, TH>(fp, a, P, tile);
+        if (PSI_CHECK(tile < fp.n_tiles_total, kChkTile, a.status)) fwd_tile<KMAX, DT, CH, LP, TH>(fp, a, P, hits, tile);
         if (!a.work) break;
         __syncthreads(); // every warp is done with this tile's pipeline
         if (threadIdx.x == 0) {
