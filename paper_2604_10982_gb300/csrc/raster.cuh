@@ -178,7 +178,7 @@ struct TopK {
 };
 
 // ------------------------------------------------------------ decoupled pipeline
-// A tile's list is streamed through kPS shared-memory stages of kPB records,
+// A tile's list is streamed through shared-memory stages of kPB records,
 // each transformed for the tile on its way in. The first 32 records per pixel
 // warp are brought in by the pixel warps themselves (pipe_prefill: one record
 // per thread, so a tile starts after one round of loads instead of after a
@@ -196,7 +196,6 @@ struct TopK {
 // following the stream to its end. `alive` counts the warps still in the walk
 // (the producer stops at zero). Every wait is bounded; a waiting warp is
 // suspended in hardware.
-constexpr int kPS = 4;            // stages
 constexpr int kPB = 128;          // records per stage (four 32-bit hit words per warp)
 // pixel warps of a 16 x TH tile (8x4-pixel blocks, two per block row) and the
 // CTA size with the producer warp
@@ -209,7 +208,12 @@ constexpr int kLeft = 0x7fffffff;  // released[w] of a warp that left the walk
 constexpr unsigned long long kTimerTickNs = 1024; // %globaltimer may advance in steps of a microsecond
 constexpr uint32_t kSuspendNs = 20000; // longest hardware suspension per poll of a wait
 
-struct Pipe {
+// NS stages: 4, or 3 where a fourth costs a resident CTA (with two of them
+// prefilled, each further one lets a fast warp run ahead of a slow one: 4
+// against 3 is 0.90 against 1.00 ms for the adjoint of the depth/normal maps)
+template <int NS>
+struct PipeT {
+    static constexpr int kPS = NS;
     float4 rec[kPS][kPB][kRecF4];
     uint32_t val[kPS][kPB];
     uint64_t ready[kPS]; // one arrival per pixel warp (the producer arrives for all of them)
@@ -219,14 +223,17 @@ struct Pipe {
     unsigned long long limit; // the context's wait limit (ns)
 };
 
+using Pipe = PipeT<4>;
+
 __device__ __forceinline__ int vload(const int &x) { return *reinterpret_cast<const volatile int *>(&x); }
 
 // thread 0; the caller synchronises the CTA afterwards. alive = the number of
 // pixel warps (each releases every stage once per batch), limit = wait_limit()
-__device__ __forceinline__ void pipe_init(Pipe &P, int alive, unsigned long long limit)
+template <class PP>
+__device__ __forceinline__ void pipe_init(PP &P, int alive, unsigned long long limit)
 {
     P.limit = limit;
-    for (int s = 0; s < kPS; ++s) {
+    for (int s = 0; s < PP::kPS; ++s) {
         mbar_init(&P.ready[s], alive);
     }
     for (int w = 0; w < kPixelWarps; ++w) P.released[w] = w < alive ? 0 : kLeft;
@@ -237,9 +244,10 @@ __device__ __forceinline__ void pipe_init(Pipe &P, int alive, unsigned long long
 
 // thread 0, between two tiles of a persistent CTA (after a CTA barrier):
 // retire the barriers so that pipe_init may initialise them again
-__device__ __forceinline__ void pipe_inval(Pipe &P)
+template <class PP>
+__device__ __forceinline__ void pipe_inval(PP &P)
 {
-    for (int s = 0; s < kPS; ++s) {
+    for (int s = 0; s < PP::kPS; ++s) {
         asm volatile("mbarrier.inval.shared::cta.b64 [%0];" ::"r"(smem_u32(&P.ready[s])) : "memory");
     }
 }
@@ -343,8 +351,8 @@ __device__ __forceinline__ void prefetch_record(const float4 *__restrict__ recor
 }
 
 // One record, transformed, into its place of a stage.
-template <bool LP>
-__device__ __forceinline__ void stage_record(Pipe &P, int s, int j, float4 (&r)[kRecF4], uint32_t i, int tile_x0,
+template <bool LP, class PP>
+__device__ __forceinline__ void stage_record(PP &P, int s, int j, float4 (&r)[kRecF4], uint32_t i, int tile_x0,
                                              int tile_y0)
 {
     transform_record<LP>(r, tile_x0, tile_y0);
@@ -371,8 +379,8 @@ __device__ __forceinline__ constexpr int prefill_batches() { return PW * 32 / kP
 
 // Pixel warp w of PW: its 32 records of the first batches (the same walk as
 // pipe_produce, after pipe_init is visible to the CTA).
-template <bool LP, int PW>
-__device__ __forceinline__ void pipe_prefill(Pipe &P, int w, const uint32_t *__restrict__ vals, int64_t list0, int n,
+template <bool LP, int PW, class PP>
+__device__ __forceinline__ void pipe_prefill(PP &P, int w, const uint32_t *__restrict__ vals, int64_t list0, int n,
                                              bool reverse, const float4 *__restrict__ records, int tile_x0,
                                              int tile_y0, DevStatus *st, uint32_t rec_lo, uint32_t rec_hi)
 {
@@ -396,8 +404,8 @@ __device__ __forceinline__ void pipe_prefill(Pipe &P, int w, const uint32_t *__r
 // Producer warp: stages the batches after the prefilled ones of the list
 // (entries [list0, list0+n)), forward or reverse, until all are staged or no
 // pixel warp is alive. Returns false on a timeout (status raised, abort set).
-template <bool LP, int PW>
-__device__ __forceinline__ bool pipe_produce(Pipe &P, const uint32_t *__restrict__ vals, int64_t list0, int n,
+template <bool LP, int PW, class PP>
+__device__ __forceinline__ bool pipe_produce(PP &P, const uint32_t *__restrict__ vals, int64_t list0, int n,
                                              bool reverse, const float4 *__restrict__ records, int tile_x0,
                                              int tile_y0, DevStatus *st, int site, uint32_t rec_lo, uint32_t rec_hi)
 {
@@ -420,14 +428,14 @@ __device__ __forceinline__ bool pipe_produce(Pipe &P, const uint32_t *__restrict
     bool v0 = entry(c, i0), v1 = entry(c + 1, i1);
 #pragma unroll 1
     for (; c < nb * kChunks; ++c) {
-        const int b = c / kChunks, s = b % kPS;
-        if (c % kChunks == 0 && b >= kPS) {
+        const int b = c / kChunks, s = b % PP::kPS;
+        if (c % kChunks == 0 && b >= PP::kPS) {
             // the stage's last batch must have been released by every pixel warp
             unsigned long long t0 = 0;
             while (true) {
                 if (vload(P.alive) == 0 || vload(P.abort)) return true;
                 const int done = lane < kPixelWarps ? ld_acquire_cta_shared(&P.released[lane]) : kLeft;
-                if (__reduce_min_sync(0xffffffffu, done) > b - kPS) break;
+                if (__reduce_min_sync(0xffffffffu, done) > b - PP::kPS) break;
                 const unsigned long long now = global_ns();
                 if (t0 == 0) {
                     t0 = now;
@@ -465,10 +473,11 @@ __device__ __forceinline__ bool pipe_produce(Pipe &P, const uint32_t *__restrict
 // after an abort. The answer is the same in every lane of the warp: once one
 // lane has seen the batch ready it stays ready (the stage cannot be refilled
 // before this warp releases it), so the others wait for it too.
-__device__ __forceinline__ bool pipe_wait_ready(Pipe &P, int b, DevStatus *st, int site)
+template <class PP>
+__device__ __forceinline__ bool pipe_wait_ready(PP &P, int b, DevStatus *st, int site)
 {
-    const int s = b % kPS;
-    const uint32_t par = (b / kPS) & 1;
+    const int s = b % PP::kPS;
+    const uint32_t par = (b / PP::kPS) & 1;
     bool ready = mbar_test_wait(&P.ready[s], par);
     if (!ready) {
         const unsigned long long limit = P.limit;
@@ -496,14 +505,16 @@ __device__ __forceinline__ bool pipe_wait_ready(Pipe &P, int b, DevStatus *st, i
 }
 
 // Pixel warp w: done with batch b and all before it.
-__device__ __forceinline__ void pipe_release(Pipe &P, int w, int b)
+template <class PP>
+__device__ __forceinline__ void pipe_release(PP &P, int w, int b)
 {
     __syncwarp();
     if ((threadIdx.x & 31) == 0) st_release_cta_shared(&P.released[w], b + 1);
 }
 
 // Pixel warp w: no pixel of it composites any further.
-__device__ __forceinline__ void pipe_leave(Pipe &P, int w)
+template <class PP>
+__device__ __forceinline__ void pipe_leave(PP &P, int w)
 {
     __syncwarp();
     if ((threadIdx.x & 31) == 0) {
@@ -525,8 +536,8 @@ using HitLists = uint8_t[kGroups][kPB];
 // the first `cnt` records of stage s, taking record j into group g's list
 // only if j < lim[g]; n[g] = length. NG = 4: one list per group; NG = 1: one
 // list (0) for the whole warp. One record per lane; every lane gets n.
-template <bool LP, int NG>
-__device__ __forceinline__ void build_hits(const Pipe &P, int s, int cnt, int vw, int tile_x0, int tile_y0,
+template <bool LP, int NG, class PP>
+__device__ __forceinline__ void build_hits(const PP &P, int s, int cnt, int vw, int tile_x0, int tile_y0,
                                            const int lim[NG], HitLists &list, int n[NG])
 {
     const int lane = threadIdx.x & 31;

@@ -283,7 +283,7 @@ __device__ __forceinline__ void bwd_tile(const FrameParams &fp, const BwdArgs &a
         if (!in_walk) pipe_leave(P, wid);
         for (int b = 0; b < nb && in_walk; ++b) {
             if (!pipe_wait_ready(P, b, a.status, kSiteRenderBwdA)) break;
-            const int st = b % kPS;
+            const int st = b % Pipe::kPS;
             int cnt;
             const int lo = batch_range(b, n, false, cnt);
             int ng[kGroups];
@@ -369,7 +369,7 @@ __device__ __forceinline__ void bwd_tile(const FrameParams &fp, const BwdArgs &a
         if (vload(P.abort)) return;
         if (tid == 0) {
             // fresh barriers for the reverse walk
-            for (int s = 0; s < kPS; ++s) {
+            for (int s = 0; s < Pipe::kPS; ++s) {
                 asm volatile("mbarrier.inval.shared::cta.b64 [%0];" ::"r"(smem_u32(&P.ready[s])) : "memory");
             }
             pipe_init(P, PW, P.limit);
@@ -408,7 +408,7 @@ __device__ __forceinline__ void bwd_tile(const FrameParams &fp, const BwdArgs &a
     const bool want_feat = !ext_feat && a.g_F && a.g_feat;
     for (int b = 0; b < nbB; ++b) {
         if (!pipe_wait_ready(P, b, a.status, kSiteRenderBwdB)) break;
-        const int st = b % kPS;
+        const int st = b % Pipe::kPS;
         int cnt;
         const int lo = batch_range(b, maxlast, true, cnt);
         int ng[NG], lim[NG];
@@ -680,7 +680,7 @@ __device__ __forceinline__ void bwd_tile_pair(const FrameParams &fp, const BwdAr
     const int nbB = (maxlast + kPB - 1) / kPB;
     for (int b = 0; b < nbB; ++b) {
         if (!pipe_wait_ready(P, b, a.status, kSiteRenderBwdB)) break;
-        const int st = b % kPS;
+        const int st = b % Pipe::kPS;
         int cnt;
         const int lo = batch_range(b, maxlast, true, cnt);
         const int limit = min(cnt, warp_last - lo); // entries [0, limit) of the batch can matter

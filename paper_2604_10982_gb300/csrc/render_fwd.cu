@@ -5,12 +5,10 @@
 // warp lists, per group of eight pixels, the records that can reach the group
 // and every group walks its own list. Per pixel (Sec. 3.1, Eq. 1): alpha =
 // min(0.99, o exp(-(u^2+v^2)/2)), RGB blended densely front to back with FP32
-// transmittance T, and the K largest weights omega_j = alpha_j T_j kept in
-// registers (Sec. 5, Top-K Hard Selection): the insertion runs under a
-// warp vote, so lanes pay one compare per surfel unless some lane of the warp
-// improves its set. After the walk the K selected features are gathered with
-// 16-byte vector loads and summed in list order in FP32:
-// F = scale * sum_{j in K} omega_j q_j.
+// transmittance T, and the K largest weights omega_j = alpha_j T_j kept
+// (Sec. 5, Top-K Hard Selection; TopK, TopKShared). After the walk
+// the K selected features are gathered row by row and summed in list order in
+// FP32: F = scale * sum_{j in K} omega_j q_j (gather_rows).
 // Dense features (K = 0) accumulate 32 channels per pass over the list.
 #include "raster.cuh"
 
@@ -41,11 +39,219 @@ struct FwdArgs {
     unsigned int *work; // persistent launch: the context's tile counter pair; NULL: one tile per CTA
 };
 
+// 16 bytes of a feature row as CPL float32 values' products with a weight:
+// acc[c] = fma(w, f_c, acc[c]), channel pairs by packed FMAs (each lane
+// rounded as the scalar one).
+template <int DT>
+__device__ __forceinline__ void fma_row(const uint4 v, float w, float2 *acc)
+{
+    const uint32_t x[4] = {v.x, v.y, v.z, v.w};
+    if constexpr (DT == PSI_F32) {
+        const float2 ww = make_float2(w, w);
+#pragma unroll
+        for (int k = 0; k < 2; ++k)
+            acc[k] = __ffma2_rn(ww, make_float2(__uint_as_float(x[2 * k]), __uint_as_float(x[2 * k + 1])), acc[k]);
+    } else if constexpr (DT == PSI_BF16) {
+        const float2 ww = make_float2(w, w);
+#pragma unroll
+        for (int k = 0; k < 4; ++k)
+            acc[k] = __ffma2_rn(ww, make_float2(__uint_as_float(x[k] << 16), __uint_as_float(x[k] & 0xFFFF0000u)), acc[k]);
+    } else {
+        // FP8 E4M3: the byte's sign at bit 31 and its 7 magnitude bits at bits
+        // [20, 27) are the value times 2^-120 (a shift that copies the sign
+        // down, the copies masked off); the weight carries the 2^120, so the
+        // product is the exact one of the decoded value
+        const float ws = w * 0x1p120f;
+        const float2 ww = make_float2(ws, ws);
+        auto val = [](uint32_t top) { return __uint_as_float(static_cast<uint32_t>(static_cast<int32_t>(top) >> 4) & 0x87F00000u); };
+#pragma unroll
+        for (int k = 0; k < 4; ++k) {
+            acc[2 * k] = __ffma2_rn(ww, make_float2(val(x[k] << 24), val(x[k] << 16)), acc[2 * k]);
+            acc[2 * k + 1] = __ffma2_rn(ww, make_float2(val(x[k] << 8), val(x[k])), acc[2 * k + 1]);
+        }
+    }
+}
+
+// The K largest weights of one pixel with their list positions (Sec. 5, Top-K
+// Hard Selection), in shared memory: slot c of a lane is the float2 (weight,
+// position bits) c & 1 of the float4 at [c >> 1][lane]. The first K weights
+// are appended, which is most of what a pixel ever keeps, so a new surfel costs one
+// store; after that a weight larger than the smallest kept one takes its
+// slot and the new smallest is looked up. Ties favour the earlier position:
+// among equal smallest weights the latest is replaced, and only by a strictly
+// larger one. In registers (TopK: sorted, shifted on every insertion) the set
+// costs 5 instructions per slot whenever any lane of the warp improves its own
+// -- nearly always while sets fill -- and K = 16 leaves room for two CTAs per
+// SM instead of three. For K <= 8 the registers are the better place (1.52
+// against 1.60 ms for the 3M-surfel 1080p frame).
+struct TopKShared {
+    int cnt, cmin; // entries; slot of the smallest
+    float wmin;    // the smallest weight
+    bool replaced; // some entry is out of list order
+
+    __device__ __forceinline__ void init()
+    {
+        cnt = cmin = 0;
+        wmin = __int_as_float(0x7f800000);
+        replaced = false;
+    }
+
+    __device__ __forceinline__ void offer(float4 *ent, int lane, int K, float w, int pos)
+    {
+        float2 *e2 = reinterpret_cast<float2 *>(ent) + 2 * lane;
+        if (cnt < K) {
+            e2[64 * (cnt >> 1) + (cnt & 1)] = make_float2(w, __int_as_float(pos));
+            if (w <= wmin) {
+                wmin = w;
+                cmin = cnt;
+            }
+            ++cnt;
+        } else if (w > wmin) {
+            e2[64 * (cmin >> 1) + (cmin & 1)] = make_float2(w, __int_as_float(pos));
+            replaced = true;
+            wmin = __int_as_float(0x7f800000);
+            int pmin = -1;
+#pragma unroll 4
+            for (int c = 0; c < K; ++c) {
+                const float2 e = e2[64 * (c >> 1) + (c & 1)];
+                const int pc = __float_as_int(e.y);
+                if (e.x < wmin || (e.x == wmin && pc > pmin)) {
+                    wmin = e.x;
+                    pmin = pc;
+                    cmin = c;
+                }
+            }
+        }
+    }
+};
+
+// float4 of shared memory per warp for the sets: K rounded up to four slots
+__host__ __device__ inline int topk_entries(int K) { return (K + 3) / 4 * 64; }
+
+// The Top-K feature sum of the warp's 32 pixels, F = scale * sum_{j in K}
+// omega_j q_j, and / or its channel argmax. ent holds each pixel's selection
+// in list order as (surfel, weight) pairs, two slots to a float4 at [slot / 2]
+// [lane], weight -1 past its end. Rows are read by whole lanes' worths of 16
+// bytes: D * esize / 16 lanes share one pixel, so the warp works on 32 / lanes
+// pixels at a time, every load covers whole rows and every store a whole row
+// of F; the kernel is bound by instruction issue, and this costs one address,
+// one load and the packed FMAs per 16 bytes of a row. (One pixel per lane,
+// 32 bytes of 32 different rows per load, was bound by the L1's tag lookups
+// and, in FP8, by five instructions per value to decode.) The order of the
+// additions is that of one lane summing alone in list order.
+template <int KMAX, int DT>
+__device__ __forceinline__ void gather_rows(const ViewParams &cam, const FwdArgs &a, int vw, int tile_x0, int tile_y0,
+                                            int K, const float4 *ent, float T)
+{
+    constexpr int CPL = DT == PSI_F32 ? 4 : (DT == PSI_BF16 ? 8 : 16); // channels per lane: 16 bytes
+    const int lane = threadIdx.x & 31;
+    const int row_lanes = a.D / CPL; // 1 .. 64
+    int lp = 1;                      // lanes per pixel: row_lanes rounded up to a power of two, at most 32
+    while (lp < row_lanes && lp < 32) lp <<= 1;
+    const int sub = lane & (lp - 1);
+    const int row_bytes = row_lanes * 16;
+#pragma unroll 1
+    for (int t = 0; t < lp; ++t) {
+        const int src = t * (32 / lp) + lane / lp; // the lane whose pixel this lane works on
+        int lxi, lyi;
+        pixel_of_thread(vw * 32 + src, lxi, lyi);
+        const int px = tile_x0 + lxi, py = tile_y0 + lyi;
+        const bool in = px < cam.W && py < cam.H;
+        const int64_t pix = cam.pix_base + static_cast<int64_t>(py) * cam.W + px;
+        float best = -__int_as_float(0x7f800000);
+        int arg = 0;
+#pragma unroll 1
+        for (int cb = 0; cb < row_lanes; cb += 32) {
+            const bool on = cb + sub < row_lanes;
+            // lanes past the row read its last 16 bytes and drop them
+            const unsigned char *base = static_cast<const unsigned char *>(a.feat) + 16 * min(cb + sub, row_lanes - 1);
+            float2 acc[CPL / 2];
+#pragma unroll
+            for (int c = 0; c < CPL / 2; ++c) acc[c] = make_float2(0.0f, 0.0f);
+#pragma unroll
+            for (int s0 = 0; s0 < KMAX; s0 += 4) {
+                if (s0 >= K) break;
+                float4 e[2];
+                e[0] = ent[(s0 / 2) * 32 + src];
+                e[1] = ent[(s0 / 2 + 1) * 32 + src];
+                // selections are packed: nothing further if no pixel has this slot
+                if (!__any_sync(0xffffffffu, e[0].y >= 0.0f)) break;
+                uint4 v[4];
+                v[0] = __ldg(reinterpret_cast<const uint4 *>(base + static_cast<int64_t>(__float_as_int(e[0].x)) * row_bytes));
+                v[1] = __ldg(reinterpret_cast<const uint4 *>(base + static_cast<int64_t>(__float_as_int(e[0].z)) * row_bytes));
+                v[2] = __ldg(reinterpret_cast<const uint4 *>(base + static_cast<int64_t>(__float_as_int(e[1].x)) * row_bytes));
+                v[3] = __ldg(reinterpret_cast<const uint4 *>(base + static_cast<int64_t>(__float_as_int(e[1].z)) * row_bytes));
+                if (e[0].y >= 0.0f) fma_row<DT>(v[0], e[0].y, acc);
+                if (e[0].w >= 0.0f) fma_row<DT>(v[1], e[0].w, acc);
+                if (e[1].y >= 0.0f) fma_row<DT>(v[2], e[1].y, acc);
+                if (e[1].w >= 0.0f) fma_row<DT>(v[3], e[1].w, acc);
+            }
+            const int c0 = (cb + sub) * CPL;
+            if (on && in) {
+                float f[CPL];
+#pragma unroll
+                for (int c = 0; c < CPL / 2; ++c) {
+                    f[2 * c] = acc[c].x;
+                    f[2 * c + 1] = acc[c].y;
+                }
+                if (a.fscale) {
+#pragma unroll
+                    for (int c = 0; c < CPL; ++c) f[c] *= __ldg(a.fscale + c0 + c);
+                }
+                if (a.F) {
+                    if (a.F_bf16) {
+                        uint32_t h[CPL / 2];
+#pragma unroll
+                        for (int c = 0; c < CPL / 2; ++c) {
+                            const __nv_bfloat162 p2 = __floats2bfloat162_rn(f[2 * c], f[2 * c + 1]);
+                            h[c] = *reinterpret_cast<const uint32_t *>(&p2);
+                        }
+                        __nv_bfloat16 *dst = static_cast<__nv_bfloat16 *>(a.F) + pix * a.D + c0;
+                        if constexpr (CPL == 4) {
+                            *reinterpret_cast<uint2 *>(dst) = make_uint2(h[0], h[1]);
+                        } else {
+#pragma unroll
+                            for (int k = 0; k < CPL / 8; ++k)
+                                reinterpret_cast<uint4 *>(dst)[k] = make_uint4(h[4 * k], h[4 * k + 1], h[4 * k + 2], h[4 * k + 3]);
+                        }
+                    } else {
+                        float4 *dst = reinterpret_cast<float4 *>(static_cast<float *>(a.F) + pix * a.D + c0);
+#pragma unroll
+                        for (int k = 0; k < CPL / 4; ++k)
+                            dst[k] = make_float4(f[4 * k], f[4 * k + 1], f[4 * k + 2], f[4 * k + 3]);
+                    }
+                }
+                if (a.argmax) {
+#pragma unroll
+                    for (int c = 0; c < CPL; ++c)
+                        if (f[c] > best) {
+                            best = f[c];
+                            arg = c0 + c;
+                        }
+                }
+            }
+        }
+        if (a.argmax) {
+            // largest value of the pixel's lanes, lowest channel on ties
+            for (int o = lp >> 1; o > 0; o >>= 1) {
+                const float ob = __shfl_xor_sync(0xffffffffu, best, o);
+                const int oa = __shfl_xor_sync(0xffffffffu, arg, o);
+                if (ob > best || (ob == best && oa < arg)) {
+                    best = ob;
+                    arg = oa;
+                }
+            }
+            const float Tp = __shfl_sync(0xffffffffu, T, src);
+            if (in && sub == 0) a.argmax[pix] = (1.0f - Tp < 1e-4f) ? -1 : arg;
+        }
+    }
+}
+
 // One tile of the frame (the whole CTA; P freshly initialised by thread 0
 // below). TH: tile height (16x16 or 16x8 tiles).
-template <int KMAX, int DT, int CH, bool LP, int TH>
-__device__ __forceinline__ void fwd_tile(const FrameParams &fp, const FwdArgs &a, Pipe &P, HitLists *hits,
-                                         uint32_t tile)
+template <int KMAX, int DT, int CH, bool LP, int TH, class PP>
+__device__ __forceinline__ void fwd_tile(const FrameParams &fp, const FwdArgs &a, PP &P, HitLists *hits,
+                                         float4 *entries, uint32_t tile)
 {
     constexpr int PW = pixel_warps(TH);
     const int tid = threadIdx.x, wid = tid >> 5, lane = tid & 31;
@@ -88,8 +294,13 @@ __device__ __forceinline__ void fwd_tile(const FrameParams &fp, const FwdArgs &a
     float T = 1.0f, cr = 0.0f, cg = 0.0f, cb = 0.0f;
     int last = 0;
     bool done = !inside;
-    TopK<(KMAX > 0 ? KMAX : 1)> top;
+    // K <= 8: sorted in registers (top); larger K: in shared memory (set)
+    constexpr bool kShared = KMAX > 8;
+    TopK<(KMAX > 0 && !kShared ? KMAX : 1)> top;
     top.init(K);
+    TopKShared set;
+    set.init();
+    float4 *ent = entries + wid * topk_entries(K);
     float facc[KMAX == 0 ? CH : 1];
 #pragma unroll
     for (int c = 0; c < (KMAX == 0 ? CH : 1); ++c) facc[c] = 0.0f;
@@ -98,7 +309,7 @@ __device__ __forceinline__ void fwd_tile(const FrameParams &fp, const FwdArgs &a
     if (!in_walk) pipe_leave(P, wid);
     for (int b = 0; b < nb && in_walk; ++b) {
         if (!pipe_wait_ready(P, b, a.status, kSiteRenderFwd)) break;
-        const int st = b % kPS;
+        const int st = b % PP::kPS;
         int cnt;
         const int lo = batch_range(b, n, false, cnt);
         // only the records that can reach a pixel of this lane's group, in list order
@@ -131,8 +342,9 @@ __device__ __forceinline__ void fwd_tile(const FrameParams &fp, const FwdArgs &a
                     }
                 }
             }
-            if constexpr (KMAX > 0) top.offer(hit, w, pos);
+            if constexpr (KMAX > 0 && !kShared) top.offer(hit, w, pos);
             if (hit) {
+                if constexpr (kShared) set.offer(ent, lane, K, w, pos);
                 T = __fmul_rn(T, __fsub_rn(1.0f, e.alpha));
                 last = pos + 1;
                 if (T < fp.t_eps) done = true;
@@ -146,10 +358,9 @@ __device__ __forceinline__ void fwd_tile(const FrameParams &fp, const FwdArgs &a
         }
     }
     if (vload(P.abort)) return;
-    if (!inside) return;
 
     const int64_t pix = cam.pix_base + static_cast<int64_t>(py) * cam.W + px;
-    if (a.write_rgb) {
+    if (inside && a.write_rgb) {
         a.rgb[pix] = cr;
         a.rgb[fp.n_pix_total + pix] = cg;
         a.rgb[2 * fp.n_pix_total + pix] = cb;
@@ -158,58 +369,53 @@ __device__ __forceinline__ void fwd_tile(const FrameParams &fp, const FwdArgs &a
     }
 
     if constexpr (KMAX == 0) {
-        if (a.F && a.feat) store_feat<CH>(a.F, a.F_bf16 != 0, pix, a.D, a.c0, facc, a.fscale);
+        if (inside && a.F && a.feat) store_feat<CH>(a.F, a.F_bf16 != 0, pix, a.D, a.c0, facc, a.fscale);
     } else {
-        top.sort_by_pos();
-        int32_t sid[KMAX];
+        TopK<KMAX> sel; // the set in list order (empty slots last)
+        if constexpr (kShared) {
+#pragma unroll
+            for (int s = 0; s < KMAX; ++s) {
+                const bool ok = s < K && s < set.cnt;
+                const float2 e = ok ? reinterpret_cast<const float2 *>(ent)[64 * (s >> 1) + 2 * lane + (s & 1)]
+                                    : make_float2(-1.0f, __int_as_float(0x7fffffff));
+                sel.w[s] = e.x;
+                sel.p[s] = __float_as_int(e.y);
+            }
+            if (__any_sync(0xffffffffu, set.replaced)) sel.sort_by_pos();
+        } else {
+            sel = top;
+            sel.sort_by_pos();
+        }
 #pragma unroll
         for (int s = 0; s < KMAX; ++s) {
-            sid[s] = top.valid(s, K) ? static_cast<int32_t>(static_cast<int64_t>(a.vals[list0 + top.p[s]]) - surf0) : -1;
-            if (!PSI_CHECK(sid[s] >= -1 && sid[s] < fp.n, kChkFeatRow, a.status)) sid[s] = -1;
+            int32_t id = sel.valid(s, K) ? static_cast<int32_t>(static_cast<int64_t>(a.vals[list0 + sel.p[s]]) - surf0) : -1;
+            if (!PSI_CHECK(id >= -1 && id < fp.n, kChkFeatRow, a.status)) id = -1;
+            sel.p[s] = id;
         }
-        if (a.topk_ids) {
+        if (inside && a.topk_ids) {
             int32_t *dst = a.topk_ids + pix * K;
 #pragma unroll
             for (int s = 0; s < KMAX; ++s)
-                if (s < K) dst[s] = sid[s];
+                if (s < K) dst[s] = sel.p[s];
         }
-        if (a.topk_w) {
+        if (inside && a.topk_w) {
             float *dst = a.topk_w + pix * K;
 #pragma unroll
             for (int s = 0; s < KMAX; ++s)
-                if (s < K) dst[s] = sid[s] >= 0 ? top.w[s] : 0.0f;
+                if (s < K) dst[s] = sel.p[s] >= 0 ? sel.w[s] : 0.0f;
         }
         if ((a.F || a.argmax) && a.feat) {
-            // 16 channels per chunk keeps the gather's registers low (one
-            // 32-byte BF16 row slice = two 16-byte loads per selected surfel)
-            constexpr int CB = 16;
-            float best = -__int_as_float(0x7f800000);
-            int arg = 0;
-            for (int c0 = 0; c0 < a.D; c0 += CB) {
-                float acc[CB];
+            auto pair = [&](int s) {
+                return make_float2(__int_as_float(max(sel.p[s], 0)), sel.p[s] >= 0 ? sel.w[s] : -1.0f);
+            };
 #pragma unroll
-                for (int c = 0; c < CB; ++c) acc[c] = 0.0f;
-#pragma unroll
-                for (int s = 0; s < KMAX; ++s) {
-                    if (sid[s] < 0) continue;
-                    float f[CB];
-                    load_feat<DT, CB>(a.feat, sid[s], a.D, c0, f, a.wide);
-#pragma unroll
-                    for (int c = 0; c < CB; ++c) acc[c] = __fmaf_rn(top.w[s], f[c], acc[c]);
+            for (int s = 0; s < KMAX; s += 2)
+                if (s < (K + 3) / 4 * 4) {
+                    const float2 e0 = pair(s), e1 = pair(s + 1);
+                    ent[(s >> 1) * 32 + lane] = make_float4(e0.x, e0.y, e1.x, e1.y);
                 }
-                if (a.F) store_feat<CB>(a.F, a.F_bf16 != 0, pix, a.D, c0, acc, a.fscale);
-                if (a.argmax) {
-#pragma unroll
-                    for (int c = 0; c < CB; ++c) {
-                        const float val = a.fscale ? acc[c] * __ldg(a.fscale + c0 + c) : acc[c];
-                        if (val > best) {
-                            best = val;
-                            arg = c0 + c;
-                        }
-                    }
-                }
-            }
-            if (a.argmax) a.argmax[pix] = (1.0f - T < 1e-4f) ? -1 : arg;
+            __syncwarp();
+            gather_rows<KMAX, DT>(cam, a, vw, tx * kTile, ty * TH - oy, K, ent, T);
         }
     }
 }
@@ -224,14 +430,15 @@ template <int KMAX, int DT, int CH, bool LP, int OCC, int TH = 16>
 __global__ void __launch_bounds__(pipe_threads(TH), OCC)
     render_fwd_kernel(const __grid_constant__ FrameParams fp, FwdArgs a)
 {
-    __shared__ __align__(128) Pipe P;
+    __shared__ __align__(128) PipeT<(KMAX > 8 ? 3 : 4)> P;
     __shared__ HitLists hits[pixel_warps(TH)];
     __shared__ uint32_t s_next;
+    extern __shared__ __align__(16) float4 entries[]; // topk_entries(K) per pixel warp
     uint32_t i = blockIdx.x;
     while (true) {
         const uint32_t tile = a.ranges[2 * fp.n_tiles_total + i];
         // debug builds: the launch order must name a tile of the frame (uniform for the CTA)
-        if (PSI_CHECK(tile < fp.n_tiles_total, kChkTile, a.status)) fwd_tile<KMAX, DT, CH, LP, TH>(fp, a, P, hits, tile);
+        if (PSI_CHECK(tile < fp.n_tiles_total, kChkTile, a.status)) fwd_tile<KMAX, DT, CH, LP, TH>(fp, a, P, hits, entries, tile);
         if (!a.work) break;
         __syncthreads(); // every warp is done with this tile's pipeline
         if (threadIdx.x == 0) {
@@ -251,18 +458,29 @@ __global__ void __launch_bounds__(pipe_threads(TH), OCC)
     }
 }
 
+template <int KMAX, int DT, int CH, bool LP, int OCC, int TH>
+cudaError_t launch_one(const FrameParams &fp, const FwdArgs &a, cudaStream_t st)
+{
+    const auto kernel = render_fwd_kernel<KMAX, DT, CH, LP, OCC, TH>;
+    const unsigned grid = a.work ? persistent_grid(fp.n_tiles_total, OCC) : fp.n_tiles_total;
+    const size_t dyn = KMAX > 0 ? static_cast<size_t>(pixel_warps(TH)) * topk_entries(fp.top_k) * sizeof(float4) : 0;
+    if (KMAX > 0) {
+        // the sets and the stages together pass 48 KB
+        const cudaError_t e = cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, static_cast<int>(dyn));
+        if (e != cudaSuccess) return e;
+    }
+    kernel<<<grid, pipe_threads(TH), dyn, st>>>(fp, a);
+    return cudaGetLastError();
+}
+
 template <int KMAX, int CH, bool LP, int OCC, int TH = 16>
 cudaError_t launch_kclo(const FrameParams &fp, const FeatView &f, const FwdArgs &a, cudaStream_t st)
 {
-    unsigned grid = fp.n_tiles_total;
-    if (a.work) grid = persistent_grid(fp.n_tiles_total, OCC);
-    constexpr int nt = pipe_threads(TH);
     switch (f.data ? f.dtype : PSI_F32) {
-    case PSI_BF16: render_fwd_kernel<KMAX, PSI_BF16, CH, LP, OCC, TH><<<grid, nt, 0, st>>>(fp, a); break;
-    case PSI_FP8_E4M3: render_fwd_kernel<KMAX, PSI_FP8_E4M3, CH, LP, OCC, TH><<<grid, nt, 0, st>>>(fp, a); break;
-    default: render_fwd_kernel<KMAX, PSI_F32, CH, LP, OCC, TH><<<grid, nt, 0, st>>>(fp, a); break;
+    case PSI_BF16: return launch_one<KMAX, PSI_BF16, CH, LP, OCC, TH>(fp, a, st);
+    case PSI_FP8_E4M3: return launch_one<KMAX, PSI_FP8_E4M3, CH, LP, OCC, TH>(fp, a, st);
+    default: return launch_one<KMAX, PSI_F32, CH, LP, OCC, TH>(fp, a, st);
     }
-    return cudaGetLastError();
 }
 
 // 16x8 tiles (Top-K with K <= 8, no low-pass filter): 4 pixel warps, up to 5 CTAs per SM
@@ -271,9 +489,10 @@ constexpr int kOccTile8 = 5;
 template <int KMAX, int CH, bool LP>
 cudaError_t launch_kcl(const FrameParams &fp, const FeatView &f, const FwdArgs &a, bool alt, cudaStream_t st)
 {
-    // K <= 8: 3 CTAs per SM (4 as the alternative); larger K and dense: 2 (1)
-    constexpr int occ = (KMAX > 0 && KMAX <= 8) ? 3 : 2;
-    constexpr int occ_alt = (KMAX > 0 && KMAX <= 8) ? 4 : 1;
+    // CTAs per SM: K <= 8: 3 (4 as the alternative); K <= 16: 3 (2), 37 KB of
+    // stages and lists and 2 KB per slot of the sets; larger K and dense: 2 (1)
+    constexpr int occ = (KMAX > 0 && KMAX <= 16) ? 3 : 2;
+    constexpr int occ_alt = (KMAX > 0 && KMAX <= 8) ? 4 : occ - 1;
     return alt ? launch_kclo<KMAX, CH, LP, occ_alt>(fp, f, a, st) : launch_kclo<KMAX, CH, LP, occ>(fp, f, a, st);
 }
 
