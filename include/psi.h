@@ -173,7 +173,7 @@ const char *psi_last_error(const psi_ctx *ctx);
  * 4 surfel id of a selected slot, 5 a saved last position past its tile's
  * list), for PSI_ERR_TIMEOUT the code of the first wait
  * that gave up (1 render, 2/3 adjoint passes, 4-6 decode, 7 drain,
- * 8 sort); then
+ * 8 sort, 9 intersect); then
  * clears the word. */
 int psi_status_fetch(psi_ctx *ctx, psi_stream stream, int32_t *status_out, int64_t *detail);
 
@@ -241,7 +241,7 @@ int psi_project_surfels(psi_ctx *ctx, const psi_surfels *s, const psi_camera *ca
                         psi_stream stream);
 
 /* ---- a2: tile intersection and key emission (Sec. 5) -------------------
- * Exclusive scan of tiles_touched, then one (key, value) pair per (tile,
+ * Prefix sums of tiles_touched and one (key, value) pair per (tile,
  * record): key = global_tile << 32 | float bits of the camera depth, value =
  * record index; records in index order, tiles row-major within a record.
  *  keys, vals:  [capacity]; d_num_pairs: device int64 receiving the pair count

@@ -57,7 +57,8 @@ enum WaitSite {
     kSiteDecodeLoad = 5,
     kSiteDecodeMma = 6,
     kSiteDrain = 7,
-    kSiteSort = 8
+    kSiteSort = 8,
+    kSiteIntersect = 9
 };
 
 struct ViewParams {
@@ -326,12 +327,6 @@ cudaError_t launch_labels(const void *F, int64_t n, int D, const float *centres,
                           cudaStream_t st, const char **why);
 cudaError_t launch_decode(const void *F, int64_t n_pix, int D, const void *Q, int n_q, const float *T, int32_t *ids,
                           void *logits, DevStatus *status, cudaStream_t st, const char **why);
-
-// Exclusive scan of uint32 counts into uint64 offsets (reduce-then-scan,
-// spin-free). Writes the total to *d_total (uint64). ws: scan_workspace_bytes(n).
-size_t scan_workspace_bytes(int64_t n);
-cudaError_t launch_scan_u32(const uint32_t *in, unsigned long long *out, int64_t n, unsigned long long *d_total,
-                            void *ws, cudaStream_t st);
 
 constexpr size_t align_up(size_t x, size_t a) { return (x + a - 1) / a * a; }
 

@@ -284,14 +284,31 @@ __device__ __forceinline__ int cost_bucket(uint32_t len)
     return 62 - min(2 * l2 + half, 62);
 }
 
-__global__ void __launch_bounds__(1024) tile_order_kernel(const uint32_t *__restrict__ ranges, int64_t n_tiles,
-                                                          uint32_t *__restrict__ order)
+// By one CTA (ranges written before a barrier of the same kernel, or by an
+// earlier one), the tiles' lengths eight loads at a time.
+__device__ __forceinline__ void order_tiles(const uint32_t *ranges, int64_t n_tiles, uint32_t *order,
+                                            unsigned int hist[64])
 {
-    __shared__ unsigned int hist[64];
+    constexpr int kU = 8;
+    // f(tile, bucket) over all tiles
+    auto sweep = [&](auto f) {
+        for (int64_t t0 = threadIdx.x; t0 < n_tiles; t0 += static_cast<int64_t>(kU) * blockDim.x) {
+            uint32_t len[kU];
+#pragma unroll
+            for (int k = 0; k < kU; ++k) {
+                const int64_t t = t0 + static_cast<int64_t>(k) * blockDim.x;
+                len[k] = t < n_tiles ? ranges[2 * t + 1] - ranges[2 * t] : 0u;
+            }
+#pragma unroll
+            for (int k = 0; k < kU; ++k) {
+                const int64_t t = t0 + static_cast<int64_t>(k) * blockDim.x;
+                if (t < n_tiles) f(t, cost_bucket(len[k]));
+            }
+        }
+    };
     if (threadIdx.x < 64) hist[threadIdx.x] = 0;
     __syncthreads();
-    for (int64_t t = threadIdx.x; t < n_tiles; t += blockDim.x)
-        atomicAdd(&hist[cost_bucket(ranges[2 * t + 1] - ranges[2 * t])], 1u);
+    sweep([&](int64_t, int b) { atomicAdd(&hist[b], 1u); });
     __syncthreads();
     if (threadIdx.x == 0) {
         unsigned int run = 0;
@@ -302,9 +319,141 @@ __global__ void __launch_bounds__(1024) tile_order_kernel(const uint32_t *__rest
         }
     }
     __syncthreads();
-    for (int64_t t = threadIdx.x; t < n_tiles; t += blockDim.x) {
-        const unsigned int pos = atomicAdd(&hist[cost_bucket(ranges[2 * t + 1] - ranges[2 * t])], 1u);
-        order[pos] = static_cast<uint32_t>(t);
+    sweep([&](int64_t t, int b) { order[atomicAdd(&hist[b], 1u)] = static_cast<uint32_t>(t); });
+}
+
+__global__ void __launch_bounds__(1024) tile_order_kernel(const uint32_t *ranges, int64_t n_tiles, uint32_t *order)
+{
+    __shared__ unsigned int hist[64];
+    order_tiles(ranges, n_tiles, order, hist);
+}
+
+// ------------------------------------------------------------------
+// Up to kSmallPairs pairs: the whole sort, the ranges and the launch order in
+// one kernel of one CTA, the pairs held in shared memory between the passes.
+// The general path is 10 kernels and two memsets whatever the count: with the
+// one-kernel intersect this takes a preview frame of about a thousand pairs
+// from 119 to 49 us. Above 8192 pairs the one SM would hold the frame up
+// longer than the launches.
+constexpr int kSmallThreads = 1024;
+constexpr int kSmallWarps = kSmallThreads / 32;
+constexpr int kSmallItems = 8;
+constexpr int kSmallPairs = kSmallThreads * kSmallItems; // 8192
+constexpr int64_t kSmallTiles = 16384;                   // tiles ranged and ordered by the one CTA
+
+struct SmallSmem {
+    uint64_t keys[kSmallPairs];
+    uint32_t vals[kSmallPairs];
+    uint16_t warp_cnt[kSmallWarps][kBins]; // at most 32 * kSmallItems of a warp's items share a digit
+    uint32_t digit_start[kBins];
+    uint32_t warp_tot[kBins / 32];
+    unsigned int hist[64];
+};
+
+__global__ void __launch_bounds__(kSmallThreads) small_sort_kernel(uint64_t *keys, uint32_t *vals, const int64_t *d_n,
+                                                                   int64_t cap, PassPlan plan, uint32_t *ranges,
+                                                                   int64_t n_tiles, DevStatus *status)
+{
+    extern __shared__ __align__(16) unsigned char smem_raw[];
+    SmallSmem &S = *reinterpret_cast<SmallSmem *>(smem_raw);
+    const int tid = threadIdx.x, lane = tid & 31, wid = tid >> 5;
+    const uint32_t lt = (1u << lane) - 1u;
+    const int n = static_cast<int>(clamped_count(d_n, cap));
+    if (tid == 0 && *d_n > cap && status) {
+        raise_status(status, PSI_ERR_CAPACITY);
+        atomicMax(&status->required_pairs, static_cast<unsigned long long>(*d_n));
+    }
+    if (ranges)
+        for (int64_t t = tid; t < 2 * n_tiles; t += kSmallThreads) ranges[t] = 0u;
+    // item i of lane l is at wid * 32 * items + i * 32 + l; as few items per
+    // thread as the count needs, so that every warp has a share
+    const int items = (n + kSmallThreads - 1) / kSmallThreads;
+    const int first = wid * 32 * items + lane;
+    uint64_t key[kSmallItems];
+    uint32_t val[kSmallItems], rank[kSmallItems];
+#pragma unroll
+    for (int i = 0; i < kSmallItems; ++i) {
+        const int idx = first + i * 32;
+        const bool ok = i < items && idx < n;
+        key[i] = ok ? keys[idx] : 0ull;
+        val[i] = ok ? vals[idx] : 0u;
+    }
+    for (int ps = 0; ps < plan.passes; ++ps) {
+        const int shift = plan.shift[ps];
+        const uint64_t mask = (1ull << plan.bits[ps]) - 1ull;
+        for (int k = tid; k < kSmallWarps * kBins / 2; k += kSmallThreads) reinterpret_cast<uint32_t *>(&S.warp_cnt[0][0])[k] = 0;
+        __syncthreads();
+#pragma unroll
+        for (int i = 0; i < kSmallItems; ++i) {
+            if (i >= items) break;
+            const bool ok = first + i * 32 < n;
+            const uint32_t d = ok ? static_cast<uint32_t>((key[i] >> shift) & mask) : (kBins + lane);
+            const uint32_t peers = __match_any_sync(0xffffffffu, d);
+            const uint32_t before = ok ? S.warp_cnt[wid][d] : 0u;
+            __syncwarp();
+            if (ok && (peers & lt) == 0) S.warp_cnt[wid][d] = static_cast<uint16_t>(before + __popc(peers));
+            __syncwarp();
+            rank[i] = before + __popc(peers & lt);
+        }
+        __syncthreads();
+        // per digit: exclusive prefix over the warps; then over the digits
+        uint32_t cnt = 0, inc = 0;
+        if (tid < kBins) {
+#pragma unroll 8
+            for (int w = 0; w < kSmallWarps; ++w) {
+                const uint32_t c = S.warp_cnt[w][tid];
+                S.warp_cnt[w][tid] = static_cast<uint16_t>(cnt);
+                cnt += c;
+            }
+            inc = cnt;
+#pragma unroll
+            for (int o = 1; o < 32; o <<= 1) {
+                const uint32_t t = __shfl_up_sync(0xffffffffu, inc, o);
+                if (lane >= o) inc += t;
+            }
+            if (lane == 31) S.warp_tot[wid] = inc;
+        }
+        __syncthreads();
+        if (tid < kBins) {
+            uint32_t before = 0;
+            for (int w = 0; w < wid; ++w) before += S.warp_tot[w];
+            S.digit_start[tid] = before + inc - cnt;
+        }
+        __syncthreads();
+#pragma unroll
+        for (int i = 0; i < kSmallItems; ++i)
+            if (i < items && first + i * 32 < n) {
+                const uint32_t d = static_cast<uint32_t>((key[i] >> shift) & mask);
+                const uint32_t pos = S.digit_start[d] + S.warp_cnt[wid][d] + rank[i];
+                S.keys[pos] = key[i];
+                S.vals[pos] = val[i];
+            }
+        __syncthreads();
+#pragma unroll
+        for (int i = 0; i < kSmallItems; ++i)
+            if (i < items && first + i * 32 < n) {
+                key[i] = S.keys[first + i * 32];
+                val[i] = S.vals[first + i * 32];
+            }
+    }
+#pragma unroll
+    for (int i = 0; i < kSmallItems; ++i) {
+        const int idx = first + i * 32;
+        if (i >= items || idx >= n) continue;
+        keys[idx] = key[i];
+        vals[idx] = val[i];
+        if (!ranges) continue;
+        const uint64_t t = key[i] >> 32;
+        if (t >= static_cast<uint64_t>(n_tiles)) {
+            raise_status(status, PSI_ERR_INVALID_ARG);
+            continue;
+        }
+        if (idx == 0 || (S.keys[idx - 1] >> 32) != t) ranges[2 * t] = static_cast<uint32_t>(idx);
+        if (idx == n - 1 || (S.keys[idx + 1] >> 32) != t) ranges[2 * t + 1] = static_cast<uint32_t>(idx + 1);
+    }
+    if (ranges) {
+        __syncthreads();
+        order_tiles(ranges, n_tiles, ranges + 2 * n_tiles, S.hist);
     }
 }
 
@@ -328,6 +477,24 @@ cudaError_t launch_sort(uint64_t *keys, uint32_t *vals, const int64_t *d_num_pai
                         cudaStream_t st)
 {
     const int64_t cap = std::max<int64_t>(capacity, 1);
+    const int nbits = std::max(end_bit - begin_bit, 1);
+    const bool want_ranges = tile_ranges && n_tiles_total > 0;
+    if (cap <= kSmallPairs && (!want_ranges || n_tiles_total <= kSmallTiles)) {
+        PassPlan plan{};
+        plan.passes = (nbits + 7) / 8;
+        const int dbits = (nbits + plan.passes - 1) / plan.passes;
+        for (int ps = 0; ps < plan.passes; ++ps) {
+            plan.shift[ps] = begin_bit + ps * dbits;
+            plan.bits[ps] = std::min(dbits, end_bit - plan.shift[ps]);
+        }
+        const cudaError_t e = cudaFuncSetAttribute(small_sort_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize,
+                                                   static_cast<int>(sizeof(SmallSmem)));
+        if (e != cudaSuccess) return e;
+        small_sort_kernel<<<1, kSmallThreads, sizeof(SmallSmem), st>>>(keys, vals, d_num_pairs, cap, plan,
+                                                                       want_ranges ? tile_ranges : nullptr,
+                                                                       n_tiles_total, status);
+        return cudaGetLastError();
+    }
     const int64_t nparts = sort_partitions(cap);
     char *p = static_cast<char *>(ws);
     auto *alt_keys = reinterpret_cast<uint64_t *>(p);
@@ -343,7 +510,6 @@ cudaError_t launch_sort(uint64_t *keys, uint32_t *vals, const int64_t *d_num_pai
     cudaError_t e = cudaMemsetAsync(zero0, 0, static_cast<size_t>(p - zero0), st);
     if (e != cudaSuccess) return e;
 
-    const int nbits = std::max(end_bit - begin_bit, 1);
     PassPlan plan{};
     plan.passes = std::max(2, (nbits + 7) / 8);
     if (plan.passes & 1) ++plan.passes;
@@ -360,7 +526,10 @@ cudaError_t launch_sort(uint64_t *keys, uint32_t *vals, const int64_t *d_num_pai
     int dev = 0, sms = 148;
     cudaGetDevice(&dev);
     cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev);
-    const unsigned hgrid = static_cast<unsigned>(std::max<int64_t>(1, std::min<int64_t>(nparts * kItems, sms * 8)));
+    // one block per 2048 pairs: each adds passes x 256 counts to the global
+    // ones, which at a block per 256 pairs outweighed reading the keys
+    // (12 us against 4 for 230k pairs)
+    const unsigned hgrid = static_cast<unsigned>(std::max<int64_t>(1, std::min<int64_t>(2 * nparts, sms * 8)));
     hist_kernel<<<hgrid, kThreads, 0, st>>>(keys, d_num_pairs, cap, plan, hist, status);
     digit_scan_kernel<<<1, kBins, 0, st>>>(hist, plan.passes);
     uint64_t *kin = keys, *kout = alt_keys;
@@ -372,7 +541,7 @@ cudaError_t launch_sort(uint64_t *keys, uint32_t *vals, const int64_t *d_num_pai
         std::swap(kin, kout);
         std::swap(vin, vout);
     }
-    if (tile_ranges && n_tiles_total > 0) {
+    if (want_ranges) {
         e = cudaMemsetAsync(tile_ranges, 0, static_cast<size_t>(n_tiles_total) * 8, st);
         if (e != cudaSuccess) return e;
         ranges_kernel<<<static_cast<unsigned>((cap + 255) / 256), 256, 0, st>>>(keys, d_num_pairs, cap, tile_ranges,
