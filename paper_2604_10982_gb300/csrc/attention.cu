@@ -49,6 +49,7 @@ using namespace tc;
 constexpr float kChi2_99 = 9.21034037198f; // -2 ln 0.01
 constexpr float kLnB = 9.21034037198f;     // ln 10000
 constexpr float kLog2e = 1.4426950408889634f;
+constexpr int kMaxGrid = 1024;   // partial slots (>= SMs of any device this runs on)
 constexpr int kAT = 128;         // surfels per tile
 constexpr int kAThreads = 320;   // 10 warps: TMA, MMA, 4 softmax, 4 psi (warps 2, 3, 8, 9)
 constexpr uint32_t kAtom = 128u * 128u; // bytes of one 128-row x 128-byte swizzle atom column
@@ -816,105 +817,155 @@ __global__ void __launch_bounds__(kAThreads, 1)
 }
 
 // ------------------------------------------------------------------ small kernels
+// The products on the queries' side (n_q <= 128 rows, C <= 128, d <= 256) and
+// the merges of the per-CTA partials, one CTA of 512 threads per row. They are
+// bound by the latency of a thread's serial loop, so every sum is split: over
+// thread groups that are added through shared memory, or over the lanes of a
+// warp. With one or two threads looping over the 152 partials of a full grid
+// the combine took 114-122 us whatever the map's size, now 10 (C = 64) to 17
+// us (C = 128); the five kernels together 248 -> 59 us (C = 128, 100 queries)
+// and 167 -> 32 us (C = 64, 20 queries).
+constexpr int kSmallThreads = 512;
+constexpr int kSmallWarps = kSmallThreads / 32;
+
+// out(e) = sum_k term(k, e) for e < width, k < count: groups of `width`
+// (rounded up to 32) threads take every other k; red: kSmallThreads floats.
+template <class Term, class Out>
+__device__ __forceinline__ void split_sum(int count, int width, float *red, Term term, Out out)
+{
+    const int wp = (width + 31) & ~31; // <= 256: at least two groups
+    const int groups = kSmallThreads / wp;
+    const int e = threadIdx.x % wp, g = threadIdx.x / wp;
+    float acc = 0.0f;
+    if (g < groups && e < width) {
+#pragma unroll 8
+        for (int k = g; k < count; k += groups) acc += term(k, e);
+    }
+    __syncthreads(); // red may still be read by an earlier sum
+    red[threadIdx.x] = acc;
+    __syncthreads();
+    if (threadIdx.x < width) {
+        float s = 0.0f;
+        for (int q = 0; q < groups; ++q) s += red[q * wp + threadIdx.x];
+        out(static_cast<int>(threadIdx.x), s);
+    }
+    __syncthreads(); // what `out` stored in shared memory is visible
+}
+
+// out(r) = sum_e v[e] M[r * d + e], r < rows: a warp per row of M
+template <class Out>
+__device__ __forceinline__ void row_dots(const float *v, const float *M, int rows, int d, Out out)
+{
+    const int lane = threadIdx.x & 31;
+    for (int r = threadIdx.x >> 5; r < rows; r += kSmallWarps) {
+        float acc = 0.0f;
+        for (int e = lane; e < d; e += 32) acc = fmaf(v[e], M[r * d + e], acc);
+        acc = warp_sum(acc);
+        if (lane == 0) out(r, acc);
+    }
+}
+
 // qh = (Q W_Q) W_K^T / sqrt(d) in FP32 and as the padded BF16 A tile [128 x C]
 // (rows >= n_q zero); q = Q W_Q kept for the adjoint. One CTA per row.
-__global__ void __launch_bounds__(256) attn_qh_kernel(const float *Q, int n_q, const float *WQ, const float *WK, int C,
-                                                      int d, float *q, float *qh, __nv_bfloat16 *qh_bf, AttnCam cam,
-                                                      AttnCam *cam_out)
+__global__ void __launch_bounds__(kSmallThreads) attn_qh_kernel(const float *Q, int n_q, const float *WQ,
+                                                                const float *WK, int C, int d, float *q, float *qh,
+                                                                __nv_bfloat16 *qh_bf, AttnCam cam, AttnCam *cam_out)
 {
-    __shared__ float qs[256];
+    __shared__ float red[kSmallThreads], qs[256], Qs[128];
     const int i = blockIdx.x;
     if (i == 0 && threadIdx.x == 0) *cam_out = cam;
     if (i >= n_q) {
-        for (int c = threadIdx.x; c < C; c += blockDim.x) qh_bf[i * C + c] = __float2bfloat16_rn(0.0f);
+        for (int c = threadIdx.x; c < C; c += kSmallThreads) qh_bf[i * C + c] = __float2bfloat16_rn(0.0f);
         return;
     }
-    for (int e = threadIdx.x; e < d; e += blockDim.x) {
-        float acc = 0.0f;
-        for (int c = 0; c < C; ++c) acc = fmaf(Q[i * C + c], WQ[c * d + e], acc);
-        qs[e] = acc;
-        q[i * d + e] = acc;
-    }
+    for (int c = threadIdx.x; c < C; c += kSmallThreads) Qs[c] = Q[i * C + c];
     __syncthreads();
+    split_sum(C, d, red, [&](int c, int e) { return Qs[c] * WQ[c * d + e]; },
+              [&](int e, float s) {
+                  qs[e] = s;
+                  q[i * d + e] = s;
+              });
     const float inv = rsqrtf(static_cast<float>(d));
-    for (int c = threadIdx.x; c < C; c += blockDim.x) {
-        float acc = 0.0f;
-        for (int e = 0; e < d; ++e) acc = fmaf(qs[e], WK[c * d + e], acc);
-        acc *= inv;
-        qh[i * C + c] = acc;
-        qh_bf[i * C + c] = __float2bfloat16_rn(acc);
-    }
+    row_dots(qs, WK, C, d, [&](int c, float s) {
+        s *= inv;
+        qh[i * C + c] = s;
+        qh_bf[i * C + c] = __float2bfloat16_rn(s);
+    });
 }
 
 // Merge the per-CTA partials of query i: M = max_g m_g, L = sum_g l_g 2^(m_g -
 // M), O = sum_g O_g 2^(m_g - M) / L (zero without active surfels), out = O W_V.
-__global__ void __launch_bounds__(256) attn_combine_kernel(const float *part_m, const float *part_l,
-                                                           const float *part_o, int G, int C, int d, const float *WV,
-                                                           float *out, float *O, float *M, float *Linv)
+__global__ void __launch_bounds__(kSmallThreads) attn_combine_kernel(const float *part_m, const float *part_l,
+                                                                     const float *part_o, int G, int C, int d,
+                                                                     const float *WV, float *out, float *O, float *M,
+                                                                     float *Linv)
 {
-    __shared__ float os[256];
-    __shared__ float Mmax, Ls;
-    const int i = blockIdx.x;
+    __shared__ float red[kSmallThreads], os[128], scale[kMaxGrid], wm[kSmallWarps], wl[kSmallWarps];
+    const int i = blockIdx.x, lane = threadIdx.x & 31, wid = threadIdx.x >> 5;
+    const float ninf = -__int_as_float(0x7f800000);
+    float m = ninf;
+    for (int g = threadIdx.x; g < G; g += kSmallThreads) m = fmaxf(m, part_m[g * 128 + i]);
+#pragma unroll
+    for (int o = 16; o > 0; o >>= 1) m = fmaxf(m, __shfl_xor_sync(0xffffffffu, m, o));
+    if (lane == 0) wm[wid] = m;
+    __syncthreads();
+    m = ninf;
+    for (int w = 0; w < kSmallWarps; ++w) m = fmaxf(m, wm[w]);
+    float l = 0.0f;
+    for (int g = threadIdx.x; g < G; g += kSmallThreads) {
+        const float lg = part_l[g * 128 + i];
+        const float sc = lg > 0.0f ? exp2f(part_m[g * 128 + i] - m) : 0.0f; // no active surfel: nothing to add
+        scale[g] = sc;
+        l += lg > 0.0f ? lg * sc : 0.0f;
+    }
+    l = warp_sum(l);
+    if (lane == 0) wl[wid] = l;
+    __syncthreads();
+    l = 0.0f;
+    for (int w = 0; w < kSmallWarps; ++w) l += wl[w];
+    const float inv = l > 0.0f ? 1.0f / l : 0.0f;
     if (threadIdx.x == 0) {
-        float m = -__int_as_float(0x7f800000);
-        for (int g = 0; g < G; ++g) m = fmaxf(m, part_m[g * 128 + i]);
-        float l = 0.0f;
-        if (m > -__int_as_float(0x7f800000))
-            for (int g = 0; g < G; ++g)
-                if (part_l[g * 128 + i] > 0.0f) l += part_l[g * 128 + i] * exp2f(part_m[g * 128 + i] - m);
-        Mmax = m;
-        Ls = l;
         M[i] = m;
-        Linv[i] = l > 0.0f ? 1.0f / l : 0.0f;
+        Linv[i] = inv;
     }
-    __syncthreads();
-    const float m = Mmax, inv = Ls > 0.0f ? 1.0f / Ls : 0.0f;
-    for (int c = threadIdx.x; c < C; c += blockDim.x) {
-        float acc = 0.0f;
-        if (inv > 0.0f)
-            for (int g = 0; g < G; ++g) {
-                const float l = part_l[g * 128 + i];
-                if (l > 0.0f) acc += part_o[(static_cast<int64_t>(g) * 128 + i) * C + c] * exp2f(part_m[g * 128 + i] - m);
-            }
-        acc *= inv;
-        os[c] = acc;
-        O[i * C + c] = acc;
-    }
-    __syncthreads();
-    for (int e = threadIdx.x; e < d; e += blockDim.x) {
-        float acc = 0.0f;
-        for (int c = 0; c < C; ++c) acc = fmaf(os[c], WV[c * d + e], acc);
-        out[i * d + e] = acc;
-    }
+    // a partial without active surfels holds no O: it is not read
+    split_sum(G, C, red,
+              [&](int g, int c) {
+                  return scale[g] > 0.0f ? part_o[(static_cast<int64_t>(g) * 128 + i) * C + c] * scale[g] : 0.0f;
+              },
+              [&](int c, float s) {
+                  os[c] = s * inv;
+                  O[i * C + c] = s * inv;
+              });
+    split_sum(C, d, red, [&](int c, int e) { return os[c] * WV[c * d + e]; },
+              [&](int e, float s) { out[i * d + e] = s; });
 }
 
 // Adjoint set-up for query i: dO = G W_V^T, D = dO . O (the forward's
 // normalised O), dO as the padded BF16 tile (rows >= n_q zero).
-__global__ void __launch_bounds__(256) attn_bwd_prep_kernel(const float *G, int n_q, const float *WV, const float *O,
-                                                            int C, int d, float *dO, float *Dq,
-                                                            __nv_bfloat16 *dO_bf)
+__global__ void __launch_bounds__(kSmallThreads) attn_bwd_prep_kernel(const float *G, int n_q, const float *WV,
+                                                                      const float *O, int C, int d, float *dO,
+                                                                      float *Dq, __nv_bfloat16 *dO_bf)
 {
-    __shared__ float red[8];
+    __shared__ float gs[256], part[128];
     const int i = blockIdx.x;
     if (i >= n_q) {
-        for (int c = threadIdx.x; c < C; c += blockDim.x) dO_bf[i * C + c] = __float2bfloat16_rn(0.0f);
+        for (int c = threadIdx.x; c < C; c += kSmallThreads) dO_bf[i * C + c] = __float2bfloat16_rn(0.0f);
         return;
     }
-    float part = 0.0f;
-    for (int c = threadIdx.x; c < C; c += blockDim.x) {
-        float acc = 0.0f;
-        for (int e = 0; e < d; ++e) acc = fmaf(G[i * d + e], WV[c * d + e], acc);
-        dO[i * C + c] = acc;
-        dO_bf[i * C + c] = __float2bfloat16_rn(acc);
-        part = fmaf(acc, O[i * C + c], part);
-    }
-    part = warp_sum(part);
-    if ((threadIdx.x & 31) == 0) red[threadIdx.x >> 5] = part;
+    for (int e = threadIdx.x; e < d; e += kSmallThreads) gs[e] = G[i * d + e];
     __syncthreads();
-    if (threadIdx.x == 0) {
+    row_dots(gs, WV, C, d, [&](int c, float s) {
+        dO[i * C + c] = s;
+        dO_bf[i * C + c] = __float2bfloat16_rn(s);
+        part[c] = s * O[i * C + c];
+    });
+    __syncthreads();
+    if (threadIdx.x < 32) {
         float s = 0.0f;
-        for (int w = 0; w < (static_cast<int>(blockDim.x) >> 5); ++w) s += red[w];
-        Dq[i] = s;
+        for (int c = threadIdx.x; c < C; c += 32) s += part[c];
+        s = warp_sum(s);
+        if (threadIdx.x == 0) Dq[i] = s;
     }
 }
 
@@ -922,53 +973,49 @@ __global__ void __launch_bounds__(256) attn_bwd_prep_kernel(const float *G, int 
 //   dqh = sum_g dqh_g,  dq = dqh W_K / sqrt(d),  dQ = dq W_Q^T
 // (rows of dQ), then dW_Q = Q^T dq, dW_K = dqh^T q / sqrt(d), dW_V = O^T G
 // (rows c of the [C x d] gradients).
-__global__ void __launch_bounds__(256) attn_bwd_q_kernel(const float *part_dq, int G, int n_q, int C, int d,
-                                                         const float *WK, const float *WQ, float *dqh, float *dq,
-                                                         float *gQ)
+__global__ void __launch_bounds__(kSmallThreads) attn_bwd_q_kernel(const float *part_dq, int G, int C, int d,
+                                                                   const float *WK, const float *WQ, float *dqh,
+                                                                   float *dq, float *gQ)
 {
-    __shared__ float hs[256], qs[256];
+    __shared__ float red[kSmallThreads], hs[128], qs[256];
     const int i = blockIdx.x;
-    for (int c = threadIdx.x; c < C; c += blockDim.x) {
-        float acc = 0.0f;
-        for (int g = 0; g < G; ++g) acc += part_dq[(static_cast<int64_t>(g) * 128 + i) * C + c];
-        hs[c] = acc;
-        dqh[i * C + c] = acc;
-    }
-    __syncthreads();
+    split_sum(G, C, red, [&](int g, int c) { return part_dq[(static_cast<int64_t>(g) * 128 + i) * C + c]; },
+              [&](int c, float s) {
+                  hs[c] = s;
+                  dqh[i * C + c] = s;
+              });
     const float inv = rsqrtf(static_cast<float>(d));
-    for (int e = threadIdx.x; e < d; e += blockDim.x) {
-        float acc = 0.0f;
-        for (int c = 0; c < C; ++c) acc = fmaf(hs[c], WK[c * d + e], acc);
-        acc *= inv;
-        qs[e] = acc;
-        dq[i * d + e] = acc;
-    }
-    __syncthreads();
-    if (gQ)
-        for (int c = threadIdx.x; c < C; c += blockDim.x) {
-            float acc = 0.0f;
-            for (int e = 0; e < d; ++e) acc = fmaf(qs[e], WQ[c * d + e], acc);
-            gQ[i * C + c] = acc;
-        }
+    split_sum(C, d, red, [&](int c, int e) { return hs[c] * WK[c * d + e]; },
+              [&](int e, float s) {
+                  qs[e] = s * inv;
+                  dq[i * d + e] = s * inv;
+              });
+    if (gQ) row_dots(qs, WQ, C, d, [&](int c, float s) { gQ[i * C + c] = s; });
 }
 
-__global__ void __launch_bounds__(256) attn_bwd_w_kernel(const float *Q, const float *q, const float *dq,
-                                                         const float *dqh, const float *O, const float *G, int n_q,
-                                                         int C, int d, float *gWQ, float *gWK, float *gWV)
+__global__ void __launch_bounds__(kSmallThreads) attn_bwd_w_kernel(const float *Q, const float *q, const float *dq,
+                                                                   const float *dqh, const float *O, const float *G,
+                                                                   int n_q, int C, int d, float *gWQ, float *gWK,
+                                                                   float *gWV)
 {
+    __shared__ float red[kSmallThreads], col[3][128];
     const int c = blockIdx.x;
-    const float inv = rsqrtf(static_cast<float>(d));
-    for (int e = threadIdx.x; e < d; e += blockDim.x) {
-        float wq = 0.0f, wk = 0.0f, wv = 0.0f;
-        for (int i = 0; i < n_q; ++i) {
-            wq = fmaf(Q[i * C + c], dq[i * d + e], wq);
-            wk = fmaf(dqh[i * C + c], q[i * d + e], wk);
-            wv = fmaf(O[i * C + c], G[i * d + e], wv);
-        }
-        if (gWQ) gWQ[c * d + e] = wq;
-        if (gWK) gWK[c * d + e] = wk * inv;
-        if (gWV) gWV[c * d + e] = wv;
+    for (int i = threadIdx.x; i < n_q; i += kSmallThreads) {
+        col[0][i] = Q[i * C + c];
+        col[1][i] = dqh[i * C + c];
+        col[2][i] = O[i * C + c];
     }
+    __syncthreads();
+    const float inv = rsqrtf(static_cast<float>(d));
+    if (gWQ)
+        split_sum(n_q, d, red, [&](int i, int e) { return col[0][i] * dq[i * d + e]; },
+                  [&](int e, float s) { gWQ[c * d + e] = s; });
+    if (gWK)
+        split_sum(n_q, d, red, [&](int i, int e) { return col[1][i] * q[i * d + e]; },
+                  [&](int e, float s) { gWK[c * d + e] = s * inv; });
+    if (gWV)
+        split_sum(n_q, d, red, [&](int i, int e) { return col[2][i] * G[i * d + e]; },
+                  [&](int e, float s) { gWV[c * d + e] = s; });
 }
 
 // ------------------------------------------------------------------ workspace
@@ -988,7 +1035,6 @@ int attn_grid(int64_t n)
     return static_cast<int>(std::max<int64_t>(1, std::min<int64_t>(tiles, sms)));
 }
 
-constexpr int kMaxGrid = 1024; // partial slots (>= SMs of any device this runs on)
 
 AttnWs carve(void *ws, int C, int d)
 {
@@ -1055,7 +1101,7 @@ cudaError_t launch_attention(const psi_surfels &s, const void *feat, int C, cons
                              float *out, void *ws, DevStatus *status, cudaStream_t st, const char **why)
 {
     const AttnWs w = carve(ws, C, d);
-    attn_qh_kernel<<<128, 256, 0, st>>>(Q, n_q, WQ, WK, C, d, w.q, w.qh, w.qh_bf, make_cam(cam, z_near), w.cam);
+    attn_qh_kernel<<<128, kSmallThreads, 0, st>>>(Q, n_q, WQ, WK, C, d, w.q, w.qh, w.qh_bf, make_cam(cam, z_near), w.cam);
     cudaError_t e = cudaGetLastError();
     if (e != cudaSuccess) return e;
     const int64_t N = s.n;
@@ -1091,7 +1137,7 @@ cudaError_t launch_attention(const psi_surfels &s, const void *feat, int C, cons
         e = cudaGetLastError();
         if (e != cudaSuccess) return e;
     }
-    attn_combine_kernel<<<n_q, 256, 0, st>>>(w.part_m, w.part_l, w.part_o, N > 0 ? G : 0, C, d, WV, out, w.O, w.M,
+    attn_combine_kernel<<<n_q, kSmallThreads, 0, st>>>(w.part_m, w.part_l, w.part_o, N > 0 ? G : 0, C, d, WV, out, w.O, w.M,
                                              w.Linv);
     return cudaGetLastError();
 }
@@ -1101,7 +1147,7 @@ cudaError_t launch_attention_bwd(const psi_surfels &s, const void *feat, int C, 
                                  float *g_mu, void *ws, DevStatus *status, cudaStream_t st, const char **why)
 {
     const AttnWs w = carve(ws, C, d);
-    attn_bwd_prep_kernel<<<128, 256, 0, st>>>(G_out, n_q, WV, w.O, C, d, w.dO, w.Dq, w.dO_bf);
+    attn_bwd_prep_kernel<<<128, kSmallThreads, 0, st>>>(G_out, n_q, WV, w.O, C, d, w.dO, w.Dq, w.dO_bf);
     cudaError_t e = cudaGetLastError();
     if (e != cudaSuccess) return e;
     const int64_t N = s.n;
@@ -1144,8 +1190,8 @@ cudaError_t launch_attention_bwd(const psi_surfels &s, const void *feat, int C, 
         e = cudaMemsetAsync(w.part_o, 0, static_cast<size_t>(128) * C * 4, st);
         if (e != cudaSuccess) return e;
     }
-    attn_bwd_q_kernel<<<n_q, 256, 0, st>>>(w.part_o, N > 0 ? G : 1, n_q, C, d, WK, WQ, w.dqh, w.dq, gQ);
-    attn_bwd_w_kernel<<<C, 256, 0, st>>>(Q, w.q, w.dq, w.dqh, w.O, G_out, n_q, C, d, gWQ, gWK, gWV);
+    attn_bwd_q_kernel<<<n_q, kSmallThreads, 0, st>>>(w.part_o, N > 0 ? G : 1, C, d, WK, WQ, w.dqh, w.dq, gQ);
+    attn_bwd_w_kernel<<<C, kSmallThreads, 0, st>>>(Q, w.q, w.dq, w.dqh, w.O, G_out, n_q, C, d, gWQ, gWK, gWV);
     return cudaGetLastError();
 }
 
