@@ -58,7 +58,7 @@ __device__ __forceinline__ float warp_transpose_sum4(float v[4], int lane)
 }
 
 // Slot indices of a pixel's sorted set: KMAX <= 8 packs them as nibbles of
-// one word (fewer registers: four CTAs per SM fit), larger sets keep an array.
+// one word (fewer registers), larger sets keep an array.
 template <int KMAX, bool PACK = (KMAX <= 8)>
 struct SlotOrder {
     int so[KMAX];
@@ -96,9 +96,9 @@ struct SlotOrder<KMAX, true> {
 // The pixel's saved set sorted by surfel id (odd-even transposition
 // network; empty slots hold 0xffffffff and sort last), with each slot's
 // weight and its index in the saved set.
-template <int KMAX>
+template <int KMAX, class Order>
 __device__ __forceinline__ void load_sorted_set(const FrameParams &fp, const FeatBwdArgs &a, bool inside, int64_t pix,
-                                                uint32_t id[KMAX], float w[KMAX], SlotOrder<KMAX> &so)
+                                                uint32_t id[KMAX], float w[KMAX], Order &so)
 {
     const int K = fp.top_k;
     so.init();
@@ -239,21 +239,27 @@ __global__ void __launch_bounds__(256, (KMAX <= 8 && NCH == 1) ? 4 : 1) feat_bwd
     }
 }
 
-// D <= 128 and K <= 8: the warp takes its 32 pixels in two passes of 16
-// (lanes 16h .. 16h + 15, the upper and lower half of its 8x4 block). A pass
-// first loads the g_F rows of its 16 pixels into registers (lanes across
-// channels: 16 float4 per lane, all loads in flight together), then visits
-// the distinct surfels its pixels selected in ascending id; per surfel only
-// the feature row is read (the next surfel's row is requested before the
-// current one is used). omega gF goes into the surfel's dL/df as above; the
-// 16 pixels' partial dots <gF, f> are summed by one transposing butterfly
-// (one per half-row holding a selecting pixel measured slower).
-// Against the per-surfel rounds above, no g_F row is read twice.
-template <int DT>
+// D <= 128: the warp takes its 32 pixels in two passes of 16 (lanes 16h ..
+// 16h + 15, the left and right half of its 8x4 block). A pass first loads the
+// g_F rows of its 16 pixels into registers (lanes across channels: 16 float4
+// per lane, all loads in flight together), then visits the distinct surfels
+// its pixels selected in ascending id; per surfel only the feature row is read
+// (the next surfel's row is requested before the current one is used). omega gF
+// goes into the surfel's dL/df as above; the 16 pixels' partial dots <gF, f>
+// are summed by one transposing butterfly (one per half-row holding a selecting
+// pixel measured slower). No g_F row is read twice: the per-surfel rounds above
+// read it once per selected surfel (704 against 458 us for K = 16, D = 128 FP32
+// at 960x540 with 500k surfels).
+// Each pixel's set, sorted by id, waits in shared memory and is consumed
+// through an index, so that moving on to a pixel's next surfel is one load
+// whatever K is (shifting K ids and weights through registers takes the same
+// time at K = 8, 0.86 ms on the 3M-surfel 1080p frame, and has no room beyond).
+constexpr int kSetBytes = 9; // id, weight, saved slot of one set entry
+template <int DT, int KMAX>
 __global__ void __launch_bounds__(256, 2) feat_bwd_reg_kernel(const __grid_constant__ FrameParams fp, FeatBwdArgs a)
 {
-    constexpr int KMAX = 8;
-    const int tid = threadIdx.x, lane = tid & 31;
+    extern __shared__ __align__(16) unsigned char set_smem[]; // per warp [K][32] (id, weight), then [K][32] slots
+    const int tid = threadIdx.x, lane = tid & 31, wid = tid >> 5;
     const uint32_t tile = blockIdx.x;
     const int v = view_of_tile(fp, tile);
     const ViewParams &cam = fp.v[v];
@@ -266,10 +272,21 @@ __global__ void __launch_bounds__(256, 2) feat_bwd_reg_kernel(const __grid_const
     const int64_t pix = cam.pix_base + static_cast<int64_t>(min(py, cam.H - 1)) * cam.W + min(px, cam.W - 1);
     const int K = fp.top_k;
 
-    uint32_t id[KMAX];
-    float w[KMAX];
-    SlotOrder<KMAX> so;
-    load_sorted_set<KMAX>(fp, a, inside, pix, id, w, so);
+    unsigned char *mine = set_smem + static_cast<size_t>(wid) * K * 32 * kSetBytes;
+    uint2 *pairs = reinterpret_cast<uint2 *>(mine) + lane;
+    uint8_t *slots = mine + K * 32 * 8 + lane;
+    {
+        uint32_t id[KMAX];
+        float w[KMAX];
+        SlotOrder<KMAX, false> so;
+        load_sorted_set<KMAX>(fp, a, inside, pix, id, w, so);
+#pragma unroll
+        for (int s = 0; s < KMAX; ++s)
+            if (s < K) { // empty slots sort last: the first K hold the set
+                pairs[32 * s] = make_uint2(id[s], __float_as_uint(w[s]));
+                slots[32 * s] = static_cast<uint8_t>(so.so[s]);
+            }
+    }
 
     // lane l owns channels [4l, 4l + 4)
     const bool con = lane < (a.D >> 2);
@@ -283,35 +300,35 @@ __global__ void __launch_bounds__(256, 2) feat_bwd_reg_kernel(const __grid_const
         const float4 f = load_feat4<DT>(a.feat, i, a.D, 4 * lane);
         return make_float4(f.x * sc.x, f.y * sc.y, f.z * sc.z, f.w * sc.w);
     };
+    const int bx = tx * kTile + (wid & 1) * 8, by = ty * fp.tile_h + (wid >> 1) * 4; // the warp's block
 #pragma unroll 1
     for (int h = 0; h < 2; ++h) {
         const bool mine_pass = (lane >> 4) == h;
+        // pixel p of the pass: (4h + (p & 3), p >> 2) of the block (pixel_of_thread)
+        const int x0 = bx + 4 * h;
         float4 G[16];
 #pragma unroll
         for (int p = 0; p < 16; ++p) {
-            const int src = 16 * h + p;
-            const long long pL = __shfl_sync(0xffffffffu, static_cast<long long>(pix), src);
-            const int inL = __shfl_sync(0xffffffffu, inside ? 1 : 0, src);
-            G[p] = (inL && con) ? __ldg(reinterpret_cast<const float4 *>(a.g_F + pL * a.D) + lane)
-                                : make_float4(0.f, 0.f, 0.f, 0.f);
+            const int x = x0 + (p & 3), y = by + (p >> 2);
+            G[p] = (x < cam.W && y < cam.H && con)
+                       ? __ldg(reinterpret_cast<const float4 *>(a.g_F + (cam.pix_base + static_cast<int64_t>(y) * cam.W + x) * a.D) + lane)
+                       : make_float4(0.f, 0.f, 0.f, 0.f);
         }
-        uint32_t cur = __reduce_min_sync(0xffffffffu, mine_pass ? id[0] : 0xffffffffu);
+        int k = 0;
+        uint2 head = mine_pass ? pairs[0] : make_uint2(0xffffffffu, 0u); // the pixel's next surfel
+        uint32_t cur = __reduce_min_sync(0xffffffffu, head.x);
         float4 f = feat_row(cur);
         while (cur != 0xffffffffu) {
-            const bool has = mine_pass && id[0] == cur; // ids are distinct within a pixel's set
-            const float wsel = w[0];
-            const long long kdi = static_cast<long long>(pix * K + so.first());
+            const bool has = head.x == cur; // ids are distinct within a pixel's set
+            const float wsel = __uint_as_float(head.y);
+            int slot = 0;
             if (has) {
-#pragma unroll
-                for (int s = 0; s + 1 < KMAX; ++s) {
-                    id[s] = id[s + 1];
-                    w[s] = w[s + 1];
-                }
-                id[KMAX - 1] = 0xffffffffu;
-                so.pop();
+                slot = slots[32 * k];
+                ++k;
+                head = k < K ? pairs[32 * k] : make_uint2(0xffffffffu, 0u);
             }
             const uint32_t m = __ballot_sync(0xffffffffu, has) >> (16 * h);
-            const uint32_t nxt = __reduce_min_sync(0xffffffffu, mine_pass ? id[0] : 0xffffffffu);
+            const uint32_t nxt = __reduce_min_sync(0xffffffffu, head.x);
             const float4 fn = feat_row(nxt);
             float4 acc = make_float4(0.f, 0.f, 0.f, 0.f);
             float part[16];
@@ -332,8 +349,8 @@ __global__ void __launch_bounds__(256, 2) feat_bwd_reg_kernel(const __grid_const
             }
             // lane l ends with the total of the pass's pixel l >> 1
             const float tot = warp_transpose_sum16(part, lane);
-            const long long kdw = __shfl_sync(0xffffffffu, kdi, 16 * h + (lane >> 1));
-            if ((lane & 1) == 0 && ((m >> (lane >> 1)) & 1u)) a.kd[kdw] = tot;
+            const float kd = __shfl_sync(0xffffffffu, tot, 2 * (lane & 15));
+            if (has) a.kd[pix * K + slot] = kd;
             if (a.g_feat && con) atomicAdd(reinterpret_cast<float4 *>(a.g_feat + static_cast<int64_t>(cur) * a.D) + lane, acc);
             cur = nxt;
             f = fn;
@@ -353,19 +370,28 @@ cudaError_t launch_kn(const FrameParams &fp, const FeatView &f, const FeatBwdArg
     return cudaGetLastError();
 }
 
+template <int KMAX, int DT>
+cudaError_t launch_reg(const FrameParams &fp, const FeatBwdArgs &a, cudaStream_t st)
+{
+    const auto kernel = feat_bwd_reg_kernel<DT, KMAX>;
+    const size_t dyn = static_cast<size_t>(pixel_warps(fp.tile_h)) * fp.top_k * 32 * kSetBytes;
+    if (dyn > 48 * 1024) {
+        const cudaError_t e = cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, static_cast<int>(dyn));
+        if (e != cudaSuccess) return e;
+    }
+    kernel<<<static_cast<unsigned>(fp.n_tiles_total), 16 * fp.tile_h, dyn, st>>>(fp, a);
+    return cudaGetLastError();
+}
+
 template <int KMAX>
 cudaError_t launch_k(const FrameParams &fp, const FeatView &f, const FeatBwdArgs &a, cudaStream_t st)
 {
-    if (KMAX == 8 && f.dim <= 128) {
-        const unsigned grid = static_cast<unsigned>(fp.n_tiles_total);
-        switch (f.dtype) {
-        case PSI_BF16: feat_bwd_reg_kernel<PSI_BF16><<<grid, 16 * fp.tile_h, 0, st>>>(fp, a); break;
-        case PSI_FP8_E4M3: feat_bwd_reg_kernel<PSI_FP8_E4M3><<<grid, 16 * fp.tile_h, 0, st>>>(fp, a); break;
-        default: feat_bwd_reg_kernel<PSI_F32><<<grid, 16 * fp.tile_h, 0, st>>>(fp, a); break;
-        }
-        return cudaGetLastError();
+    if (f.dim > 128) return launch_kn<KMAX, 2>(fp, f, a, st);
+    switch (f.dtype) {
+    case PSI_BF16: return launch_reg<KMAX, PSI_BF16>(fp, a, st);
+    case PSI_FP8_E4M3: return launch_reg<KMAX, PSI_FP8_E4M3>(fp, a, st);
+    default: return launch_reg<KMAX, PSI_F32>(fp, a, st);
     }
-    return f.dim > 128 ? launch_kn<KMAX, 2>(fp, f, a, st) : launch_kn<KMAX, 1>(fp, f, a, st);
 }
 
 } // namespace
