@@ -222,7 +222,7 @@ int psi_view_layout(const psi_camera *cams, int n_views, const psi_render_opts *
 int psi_intersect_workspace_size(int64_t n_records, size_t *bytes);
 int psi_sort_workspace_size(int64_t capacity, size_t *bytes);
 /* Adjoint scratch: per-record moments (n_records = n_views * N) and, for
- * top_k > 0, one float per (pixel, selected slot) (n_pix = P_total). */
+ * top_k > 0, an id and a float per (pixel, selected slot) (n_pix = P_total). */
 int psi_render_bwd_workspace_size(int64_t n_records, int64_t n_pix, int top_k, size_t *bytes);
 
 /* ---- a1: projection and ray-splat setup --------------------------------
@@ -341,9 +341,10 @@ int psi_grads_zero(psi_ctx *ctx, const psi_grads *grads, int64_t n, int dim, psi
 /* ---- launch-shape autotuner for a4 and a5 (no counterpart in the paper) ---
  * The compositing kernels are compiled in PSI_RENDER_SHAPES launch shapes:
  * bit 0 of a shape builds the kernel for the other number of resident CTAs
- * per SM (top_k <= 8: forward and recomputing adjoint 3 -> 4, adjoint from
- * saved state 4 -> 3, its paired walk 4 -> 3; forward with top_k 9..16:
- * 3 -> 2; otherwise 2 -> 1), i.e. registers per
+ * per SM (adjoint from saved state with top_k 1..8 and its paired walk 4 -> 3,
+ * with top_k > 8 3 -> 4;
+ * top_k <= 8: forward and recomputing adjoint 3 -> 4; forward with top_k
+ * 9..16: 3 -> 2; otherwise 2 -> 1), i.e. registers per
  * thread against occupancy; bit 1 composites dense features
  * (top_k = 0, dim a multiple of 32) 16 channels per pass instead of 32;
  * bit 2 is the persistent launch: a few CTAs per SM, each taking tiles

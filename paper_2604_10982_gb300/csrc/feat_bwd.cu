@@ -29,7 +29,7 @@ struct FeatBwdArgs {
     const int32_t *topk_ids; // [P_total, K]
     const float *topk_w;     // [P_total, K]
     const float *g_F;        // [P_total, D]
-    float *kd;               // [P_total, K]
+    uint2 *sel;              // [P_total, K] out: (surfel id or -1, kd) per saved slot
     float *g_feat;           // [N, D] or NULL
     DevStatus *status;
 };
@@ -109,6 +109,7 @@ __device__ __forceinline__ void load_sorted_set(const FrameParams &fp, const Fea
         if (!PSI_CHECK(i >= -1 && i < fp.n, kChkFeatRow, a.status)) i = -1;
         id[s] = static_cast<uint32_t>(i);
         w[s] = i >= 0 ? a.topk_w[pix * K + s] : 0.0f;
+        if (inside && s < K && i < 0) a.sel[pix * K + s] = make_uint2(0xffffffffu, 0u);
     }
 #pragma unroll
     for (int round = 0; round < KMAX; ++round) {
@@ -229,7 +230,7 @@ __global__ void __launch_bounds__(256, (KMAX <= 8 && NCH == 1) ? 4 : 1) feat_bwd
             const float tot = warp_transpose_sum4(part, lane);
             const int myq = min(__popc(taken & lt), 3);
             const float mykd = __shfl_sync(0xffffffffu, tot, 8 * myq);
-            if ((taken >> lane) & 1u) a.kd[kdi] = mykd;
+            if ((taken >> lane) & 1u) a.sel[kdi] = make_uint2(cur, __float_as_uint(mykd));
         }
         if (a.g_feat) {
             float4 *dst = reinterpret_cast<float4 *>(a.g_feat + static_cast<int64_t>(cur) * a.D);
@@ -350,7 +351,7 @@ __global__ void __launch_bounds__(256, 2) feat_bwd_reg_kernel(const __grid_const
             // lane l ends with the total of the pass's pixel l >> 1
             const float tot = warp_transpose_sum16(part, lane);
             const float kd = __shfl_sync(0xffffffffu, tot, 2 * (lane & 15));
-            if (has) a.kd[pix * K + slot] = kd;
+            if (has) a.sel[pix * K + slot] = make_uint2(cur, __float_as_uint(kd));
             if (a.g_feat && con) atomicAdd(reinterpret_cast<float4 *>(a.g_feat + static_cast<int64_t>(cur) * a.D) + lane, acc);
             cur = nxt;
             f = fn;
@@ -397,7 +398,7 @@ cudaError_t launch_k(const FrameParams &fp, const FeatView &f, const FeatBwdArgs
 } // namespace
 
 cudaError_t launch_feat_bwd(const FrameParams &fp, const FeatView &f, const int32_t *topk_ids, const float *topk_w,
-                            const float *g_F, float *kd, float *g_feat, DevStatus *status, cudaStream_t st)
+                            const float *g_F, uint2 *sel, float *g_feat, DevStatus *status, cudaStream_t st)
 {
     if (fp.n_tiles_total == 0 || fp.top_k <= 0 || !f.data || !g_F) return cudaSuccess;
     FeatBwdArgs a{};
@@ -407,7 +408,7 @@ cudaError_t launch_feat_bwd(const FrameParams &fp, const FeatView &f, const int3
     a.topk_ids = topk_ids;
     a.topk_w = topk_w;
     a.g_F = g_F;
-    a.kd = kd;
+    a.sel = sel;
     a.g_feat = g_feat;
     a.status = status;
     if (fp.top_k <= 8) return launch_k<8>(fp, f, a, st);

@@ -68,59 +68,73 @@ struct BwdArgs {
     // forward state of the same frame (all NULL: recompute it in pass A)
     const float *saved_T;      // [P_total]
     const int32_t *saved_last; // [P_total]
-    const int32_t *saved_topk; // [P_total, K] surfel ids in list order, -1 padded
-    const float *kd_saved;     // [P_total, K] <gF, f_j> of the saved set (feat_bwd.cu), or NULL
+    const uint2 *sel;          // [P_total, K] (surfel id, <gF, f_j>) of the saved set in list order, id -1 padded
+                               // (feat_bwd.cu), or NULL
     unsigned int *work;        // persistent launch: the context's adjoint tile counter pair; NULL: one tile per CTA
 };
 
 // The saved Top-K set of one pixel met during pass B. The saved ids are in
 // list order, so walking back to front the next selected surfel the pixel
 // meets is always the last of its set not met yet: one compare per (record,
-// pixel). Keeps that id and its <gF, f>, the one after it (prefetched when
-// one is met, so its load has a whole stretch of the walk to land) and the
-// slot before that.
+// pixel). Keeps that id and its <gF, f> and the ones after it, requested when
+// one is met, so that the load has a whole stretch of the walk to land. The
+// feature kernel leaves (id, <gF, f>) side by side: one 8-byte load per met
+// surfel, through a running pointer (with the ids and the products in two
+// arrays indexed by pixel: 1.78 against 1.70 ms for the walk of the
+// 3M-surfel 1080p frame).
 struct SavedSel {
-    int nid, nnid, ptr;
+    int nid, nnid, left; // left: slots before the one of nnid
     float nkd, nnkd;
+    const uint2 *next; // the slot before the one of nnid
 
-    __device__ __forceinline__ void init(const BwdArgs &a, int64_t pix, int K, int64_t n_surf, bool on)
+    __device__ __forceinline__ void init(const BwdArgs &a, int64_t pix, int K, bool on)
     {
-        nid = nnid = ptr = -1;
+        nid = nnid = -1;
+        left = 0;
         nkd = nnkd = 0.0f;
-        if (!on || !a.kd_saved) return;
-        const int32_t *ids = a.saved_topk + pix * K;
-        const float *kds = a.kd_saved + pix * K;
-#pragma unroll 4
-        for (int s = 0; s < K; ++s) {
-            int id = ids[s];
-            // debug builds: a saved id must be -1 or a surfel of the table
-            if (!PSI_CHECK(id >= -1 && id < n_surf, kChkFeatRow, a.status)) id = -1;
-            if (id >= 0) {
-                nnid = nid;
-                nnkd = nkd;
-                nid = id;
-                nkd = kds[s];
-                ptr = s - 2;
-            }
+        next = nullptr;
+        if (!on || !a.sel) return;
+        // the set fills its first slots: its last entry from the back, four at a time
+        const uint2 *sel = a.sel + pix * K;
+        for (int s = K - 1; s >= 0 && nid < 0; s -= 4) {
+            uint2 e[4];
+#pragma unroll
+            for (int k = 0; k < 4; ++k) e[k] = s - k >= 0 ? sel[s - k] : make_uint2(0xffffffffu, 0u);
+#pragma unroll
+            for (int k = 3; k >= 0; --k) // the highest slot last
+                if (static_cast<int>(e[k].x) >= 0) {
+                    nnid = nid;
+                    nnkd = nkd;
+                    nid = static_cast<int>(e[k].x);
+                    nkd = __uint_as_float(e[k].y);
+                    left = s - k - 1;
+                }
         }
+        if (nid >= 0 && nnid < 0 && left >= 0) {
+            const uint2 e = sel[left]; // the one before it, if that was in the next four
+            nnid = static_cast<int>(e.x);
+            nnkd = __uint_as_float(e.y);
+        }
+        next = sel + (left - 1);
     }
 
     // <gF, f_sid> if sid is the pixel's next selected surfel (then advance), else 0
-    __device__ __forceinline__ float match(const BwdArgs &a, int64_t pix, int K, int64_t n_surf, int sid)
+    __device__ __forceinline__ float match(int sid)
     {
         if (sid != nid) return 0.0f;
         const float dot = nkd;
         nid = nnid;
         nkd = nnkd;
         nnid = -1;
-        nnkd = 0.0f;
-        if (ptr >= 0) {
-            int id = a.saved_topk[pix * K + ptr];
-            if (!PSI_CHECK(id >= -1 && id < n_surf, kChkFeatRow, a.status)) id = -1;
-            nnid = id;
-            nnkd = a.kd_saved[pix * K + ptr];
-        }
-        --ptr;
+        // a predicated load into the two registers, so that nothing waits for
+        // it before the pixel's next match (a branch or a select would)
+        asm volatile(
+            "{\n\t.reg .pred p;\n\tsetp.gt.s32 p, %3, 0;\n\t"
+            "@p ld.global.v2.b32 {%0, %1}, [%2];\n\t}"
+            : "+r"(nnid), "+f"(nnkd)
+            : "l"(next), "r"(left));
+        --next;
+        --left;
         return dot;
     }
 };
@@ -383,7 +397,7 @@ __device__ __forceinline__ void bwd_tile(const FrameParams &fp, const BwdArgs &a
         return;
     }
     pipe_prefill<LP, PW>(P, wid, a.vals, list0, maxlast, true, a.records, tileX, tileY, a.status, rec_lo, rec_hi);
-    if constexpr (ext_feat) sel_saved.init(a, pix, K, fp.n, inside);
+    if constexpr (ext_feat) sel_saved.init(a, pix, K, inside);
     // entries at or beyond every lane's last composited surfel are skipped by
     // the group (the warp when it walks one list)
     constexpr int NG = (ext_feat || NW) ? kGroups : 1;
@@ -452,7 +466,7 @@ __device__ __forceinline__ void bwd_tile(const FrameParams &fp, const BwdArgs &a
                         w = e.alpha * Tj;
                         float dot = 0.0f;
                         if constexpr (ext_feat) {
-                            dot = sel_saved.match(a, pix, K, fp.n, static_cast<int>(sid));
+                            dot = sel_saved.match(static_cast<int>(sid));
                         } else if constexpr (KMAX > 0) {
 #pragma unroll
                             for (int s = 0; s < KMAX; ++s)
@@ -656,7 +670,7 @@ __device__ __forceinline__ void bwd_tile_pair(const FrameParams &fp, const BwdAr
         if (!PSI_CHECK(l >= 0 && l <= n, kChkLast, a.status)) l = 0;
         last[h] = min(max(l, 0), n);
         Tc[h] = T;
-        sel[h].init(a, pix[h], K, fp.n, inside);
+        sel[h].init(a, pix[h], K, inside);
         gr[h] = inside ? a.g_rgb[pix[h]] : 0.0f;
         gg[h] = inside ? a.g_rgb[fp.n_pix_total + pix[h]] : 0.0f;
         gb[h] = inside ? a.g_rgb[2 * fp.n_pix_total + pix[h]] : 0.0f;
@@ -723,7 +737,7 @@ __device__ __forceinline__ void bwd_tile_pair(const FrameParams &fp, const BwdAr
                         const float inv = rcp_approx(one_m); // one_m >= 0.01
                         const float Tj = Tc[h] * inv;
                         const float w = e[h].alpha * Tj;
-                        const float dot = sel[h].match(a, pix[h], K, fp.n, sid);
+                        const float dot = sel[h].match(sid);
                         const float sj = gr[h] * col.y + gg[h] * col.z + gb[h] * col.w + dot;
                         const float dLda = Tj * sj - suffix[h] * inv;
                         suffix[h] = fmaf(w, sj, suffix[h]);
@@ -974,10 +988,11 @@ constexpr int kOccTile8 = 5;
 template <int KMAX, int CH, bool SAVED, bool LP>
 cudaError_t launch_kcsl(const FrameParams &fp, const FeatView &f, const BwdArgs &a, bool alt, cudaStream_t st)
 {
-    // K <= 8: 3 CTAs per SM when pass A recomputes the Top-K set (the 4-CTA
-    // build spills in the per-record reductions), 4 from saved state (56
-    // registers, no Top-K in registers); larger K (register Top-K of 16 or
-    // 32) and dense: 2 (the alternative shape: 4 resp. 3, and 1)
+    // From saved state with a selection: 4 CTAs per SM (56 registers), or the
+    // alternative 3 for K > 8; K <= 8 when pass A recomputes the set: 3
+    // (the 4-CTA build spills in the per-record reductions); larger K
+    // recomputed (register Top-K of 16 or 32) and dense: 2 (the alternative
+    // shape: 3, 4, and 1)
     constexpr bool small = KMAX > 0 && KMAX <= 8;
     constexpr int occ = small ? (SAVED ? 4 : 3) : 2;
     constexpr int occ_alt = small ? (SAVED ? 3 : 4) : 1;
@@ -1012,20 +1027,18 @@ cudaError_t launch_kcs(const FrameParams &fp, const FeatView &f, const BwdArgs &
                       : launch_kcsl<KMAX, CH, SAVED, false>(fp, f, a, alt, st);
 }
 
-template <int KMAX, int CH>
-cudaError_t launch_kc(const FrameParams &fp, const FeatView &f, const BwdArgs &a, bool alt, cudaStream_t st)
+// Recomputing walk with a Top-K selection.
+template <int KMAX>
+cudaError_t launch_recompute(const FrameParams &fp, const FeatView &f, const BwdArgs &a, bool alt, cudaStream_t st)
 {
-    return a.saved_T ? launch_kcs<KMAX, CH, true>(fp, f, a, alt, st) : launch_kcs<KMAX, CH, false>(fp, f, a, alt, st);
+    return launch_kcs<KMAX, 16, false>(fp, f, a, alt, st);
 }
 
-template <int KMAX>
-cudaError_t launch_k(const FrameParams &fp, const FeatView &f, const BwdArgs &a, int ch, bool alt, cudaStream_t st)
+// Dense features: the channel chunk shapes the feature dot product.
+template <int CH>
+cudaError_t launch_dense(const FrameParams &fp, const FeatView &f, const BwdArgs &a, bool alt, cudaStream_t st)
 {
-    // the channel chunk only shapes the dense (K = 0) feature dot product
-    if constexpr (KMAX > 0)
-        return launch_kc<KMAX, 16>(fp, f, a, alt, st);
-    else
-        return ch == 32 ? launch_kc<KMAX, 32>(fp, f, a, alt, st) : launch_kc<KMAX, 16>(fp, f, a, alt, st);
+    return a.saved_T ? launch_kcs<0, CH, true>(fp, f, a, alt, st) : launch_kcs<0, CH, false>(fp, f, a, alt, st);
 }
 
 } // namespace
@@ -1039,8 +1052,8 @@ size_t moments_bytes(int64_t n_records)
 
 size_t render_bwd_workspace_bytes(int64_t n_records, int64_t n_pix, int top_k)
 {
-    const size_t kd = top_k > 0 ? align_up(static_cast<size_t>(n_pix) * top_k * sizeof(float), 256) : 0;
-    return moments_bytes(n_records) + kd;
+    const size_t sel = top_k > 0 ? align_up(static_cast<size_t>(n_pix) * top_k * sizeof(uint2), 256) : 0;
+    return moments_bytes(n_records) + sel;
 }
 
 cudaError_t launch_render_bwd(const FrameParams &fp, const psi_surfels &s, const FeatView &f, const float4 *records,
@@ -1073,15 +1086,14 @@ cudaError_t launch_render_bwd(const FrameParams &fp, const psi_surfels &s, const
     if (saved) {
         a.saved_T = saved->T;
         a.saved_last = saved->n_last;
-        a.saved_topk = saved->topk_ids;
         if (fp.top_k > 0 && a.g_F) {
-            // feature terms from the saved selection: kd for the walk, dL/df
-            float *kd = reinterpret_cast<float *>(static_cast<char *>(ws) + moments_bytes(R));
+            // feature terms from the saved selection: <gF, f> for the walk, dL/df
+            uint2 *sel = reinterpret_cast<uint2 *>(static_cast<char *>(ws) + moments_bytes(R));
             mark(PSI_KERNEL_BWD_FEAT, 0);
-            e = launch_feat_bwd(fp, f, saved->topk_ids, saved->topk_w, a.g_F, kd, a.g_feat, status, st);
+            e = launch_feat_bwd(fp, f, saved->topk_ids, saved->topk_w, a.g_F, sel, a.g_feat, status, st);
             if (e != cudaSuccess) return e;
             mark(PSI_KERNEL_BWD_FEAT, 1);
-            a.kd_saved = kd;
+            a.sel = sel;
         }
     }
     const int K = fp.top_k;
@@ -1095,13 +1107,18 @@ cudaError_t launch_render_bwd(const FrameParams &fp, const psi_surfels &s, const
         e = a.saved_T ? launch_kcslo<8, 16, true, false, kOccTile8, 8>(fp, f, a, st)
                       : launch_kcslo<8, 16, false, false, kOccTile8, 8>(fp, f, a, st);
     else if (K == 0)
-        e = launch_k<0>(fp, f, a, ch, alt, st);
+        e = ch == 32 ? launch_dense<32>(fp, f, a, alt, st) : launch_dense<16>(fp, f, a, alt, st);
+    else if (a.saved_T)
+        // the walk from saved state keeps no set in registers: one build for
+        // every K. With K > 8 three CTAs per SM leave more of the L1 for the
+        // sets (264 against 286 us for K = 16 at 960x540, 500k surfels)
+        e = launch_kcs<8, 16, true>(fp, f, a, alt != (K > 8), st);
     else if (K <= 8)
-        e = launch_k<8>(fp, f, a, ch, alt, st);
+        e = launch_recompute<8>(fp, f, a, alt, st);
     else if (K <= 16)
-        e = launch_k<16>(fp, f, a, ch, alt, st);
+        e = launch_recompute<16>(fp, f, a, alt, st);
     else
-        e = launch_k<32>(fp, f, a, ch, alt, st);
+        e = launch_recompute<32>(fp, f, a, alt, st);
     if (e != cudaSuccess) return e;
     mark(PSI_KERNEL_BWD_WALK, 1);
     if (lp)
