@@ -818,13 +818,15 @@ __global__ void __launch_bounds__(kAThreads, 1)
 
 // ------------------------------------------------------------------ small kernels
 // The products on the queries' side (n_q <= 128 rows, C <= 128, d <= 256) and
-// the merges of the per-CTA partials, one CTA of 512 threads per row. They are
-// bound by the latency of a thread's serial loop, so every sum is split: over
-// thread groups that are added through shared memory, or over the lanes of a
-// warp. With one or two threads looping over the 152 partials of a full grid
-// the combine took 114-122 us whatever the map's size, now 10 (C = 64) to 17
-// us (C = 128); the five kernels together 248 -> 59 us (C = 128, 100 queries)
-// and 167 -> 32 us (C = 64, 20 queries).
+// the merges of the per-CTA partials, one CTA of 512 threads per row; bound by
+// the latency of serial sums. What is rounded to BF16 further on, or scales
+// what is (qh, the forward's sum and O, dO, D), keeps the order of one serial
+// sum -- a different last bit there moves BF16 roundings of the large kernels --
+// and gets its operands faster: staged through shared memory, or many loads
+// ahead. The other sums are split over thread groups or the lanes of a warp.
+// With one thread walking global memory per sum the combine took 114-122 us
+// whatever the map's size, now 19; the five kernels together 167 -> 38 us (C =
+// 64, 20 queries).
 constexpr int kSmallThreads = 512;
 constexpr int kSmallWarps = kSmallThreads / 32;
 
@@ -865,13 +867,31 @@ __device__ __forceinline__ void row_dots(const float *v, const float *M, int row
     }
 }
 
+// The same in the order e = 0, 1, .. of one serial sum per row (rows <= 128):
+// M passes through shared memory 32 columns at a time; tile: 128 x 33 floats.
+template <class Out>
+__device__ __forceinline__ void row_dots_serial(const float *v, const float *M, int rows, int d, float *tile, Out out)
+{
+    float acc = 0.0f;
+    for (int e0 = 0; e0 < d; e0 += 32) {
+        const int m = min(32, d - e0);
+        for (int k = threadIdx.x; k < rows * 32; k += kSmallThreads)
+            if ((k & 31) < m) tile[(k >> 5) * 33 + (k & 31)] = M[(k >> 5) * d + e0 + (k & 31)];
+        __syncthreads();
+        if (threadIdx.x < rows)
+            for (int k = 0; k < m; ++k) acc = fmaf(v[e0 + k], tile[threadIdx.x * 33 + k], acc);
+        __syncthreads();
+    }
+    if (threadIdx.x < rows) out(static_cast<int>(threadIdx.x), acc);
+}
+
 // qh = (Q W_Q) W_K^T / sqrt(d) in FP32 and as the padded BF16 A tile [128 x C]
 // (rows >= n_q zero); q = Q W_Q kept for the adjoint. One CTA per row.
 __global__ void __launch_bounds__(kSmallThreads) attn_qh_kernel(const float *Q, int n_q, const float *WQ,
                                                                 const float *WK, int C, int d, float *q, float *qh,
                                                                 __nv_bfloat16 *qh_bf, AttnCam cam, AttnCam *cam_out)
 {
-    __shared__ float red[kSmallThreads], qs[256], Qs[128];
+    __shared__ float tile[128 * 33], qs[256], Qs[128];
     const int i = blockIdx.x;
     if (i == 0 && threadIdx.x == 0) *cam_out = cam;
     if (i >= n_q) {
@@ -880,13 +900,16 @@ __global__ void __launch_bounds__(kSmallThreads) attn_qh_kernel(const float *Q, 
     }
     for (int c = threadIdx.x; c < C; c += kSmallThreads) Qs[c] = Q[i * C + c];
     __syncthreads();
-    split_sum(C, d, red, [&](int c, int e) { return Qs[c] * WQ[c * d + e]; },
-              [&](int e, float s) {
-                  qs[e] = s;
-                  q[i * d + e] = s;
-              });
+    for (int e = threadIdx.x; e < d; e += kSmallThreads) {
+        float acc = 0.0f;
+#pragma unroll 16
+        for (int c = 0; c < C; ++c) acc = fmaf(Qs[c], WQ[c * d + e], acc);
+        qs[e] = acc;
+        q[i * d + e] = acc;
+    }
+    __syncthreads();
     const float inv = rsqrtf(static_cast<float>(d));
-    row_dots(qs, WK, C, d, [&](int c, float s) {
+    row_dots_serial(qs, WK, C, d, tile, [&](int c, float s) {
         s *= inv;
         qh[i * C + c] = s;
         qh_bf[i * C + c] = __float2bfloat16_rn(s);
@@ -900,7 +923,7 @@ __global__ void __launch_bounds__(kSmallThreads) attn_combine_kernel(const float
                                                                      const float *WV, float *out, float *O, float *M,
                                                                      float *Linv)
 {
-    __shared__ float red[kSmallThreads], os[128], scale[kMaxGrid], wm[kSmallWarps], wl[kSmallWarps];
+    __shared__ float red[kSmallThreads], os[128], scale[kMaxGrid], lg[kMaxGrid], wm[kSmallWarps], s_inv;
     const int i = blockIdx.x, lane = threadIdx.x & 31, wid = threadIdx.x >> 5;
     const float ninf = -__int_as_float(0x7f800000);
     float m = ninf;
@@ -911,32 +934,42 @@ __global__ void __launch_bounds__(kSmallThreads) attn_combine_kernel(const float
     __syncthreads();
     m = ninf;
     for (int w = 0; w < kSmallWarps; ++w) m = fmaxf(m, wm[w]);
-    float l = 0.0f;
     for (int g = threadIdx.x; g < G; g += kSmallThreads) {
-        const float lg = part_l[g * 128 + i];
-        const float sc = lg > 0.0f ? exp2f(part_m[g * 128 + i] - m) : 0.0f; // no active surfel: nothing to add
-        scale[g] = sc;
-        l += lg > 0.0f ? lg * sc : 0.0f;
+        const float l = part_l[g * 128 + i];
+        lg[g] = l;
+        scale[g] = l > 0.0f ? exp2f(part_m[g * 128 + i] - m) : 0.0f; // no active surfel: nothing to add
     }
-    l = warp_sum(l);
-    if (lane == 0) wl[wid] = l;
     __syncthreads();
-    l = 0.0f;
-    for (int w = 0; w < kSmallWarps; ++w) l += wl[w];
-    const float inv = l > 0.0f ? 1.0f / l : 0.0f;
-    if (threadIdx.x == 0) {
+    if (threadIdx.x == kSmallThreads - 32) { // a warp that holds no channel
+        float l = 0.0f;
+#pragma unroll 8
+        for (int g = 0; g < G; ++g)
+            if (lg[g] > 0.0f) l = fmaf(lg[g], scale[g], l);
+        s_inv = l > 0.0f ? 1.0f / l : 0.0f;
         M[i] = m;
-        Linv[i] = inv;
+        Linv[i] = s_inv;
     }
-    // a partial without active surfels holds no O: it is not read
-    split_sum(G, C, red,
-              [&](int g, int c) {
-                  return scale[g] > 0.0f ? part_o[(static_cast<int64_t>(g) * 128 + i) * C + c] * scale[g] : 0.0f;
-              },
-              [&](int c, float s) {
-                  os[c] = s * inv;
-                  O[i * C + c] = s * inv;
-              });
+    // meanwhile: a partial without active surfels holds no O, it is not read
+    float acc = 0.0f;
+    if (threadIdx.x < C) {
+        constexpr int kU = 16;
+        for (int g0 = 0; g0 < G; g0 += kU) {
+            float v[kU];
+#pragma unroll
+            for (int k = 0; k < kU; ++k)
+                v[k] = g0 + k < G && lg[g0 + k] > 0.0f ? part_o[(static_cast<int64_t>(g0 + k) * 128 + i) * C + threadIdx.x] : 0.0f;
+#pragma unroll
+            for (int k = 0; k < kU; ++k)
+                if (g0 + k < G && lg[g0 + k] > 0.0f) acc = fmaf(v[k], scale[g0 + k], acc);
+        }
+    }
+    __syncthreads();
+    if (threadIdx.x < C) {
+        acc *= s_inv;
+        os[threadIdx.x] = acc;
+        O[i * C + threadIdx.x] = acc;
+    }
+    __syncthreads();
     split_sum(C, d, red, [&](int c, int e) { return os[c] * WV[c * d + e]; },
               [&](int e, float s) { out[i * d + e] = s; });
 }
@@ -947,7 +980,7 @@ __global__ void __launch_bounds__(kSmallThreads) attn_bwd_prep_kernel(const floa
                                                                       const float *O, int C, int d, float *dO,
                                                                       float *Dq, __nv_bfloat16 *dO_bf)
 {
-    __shared__ float gs[256], part[128];
+    __shared__ float tile[128 * 33], gs[256], part[128], red[4];
     const int i = blockIdx.x;
     if (i >= n_q) {
         for (int c = threadIdx.x; c < C; c += kSmallThreads) dO_bf[i * C + c] = __float2bfloat16_rn(0.0f);
@@ -955,17 +988,22 @@ __global__ void __launch_bounds__(kSmallThreads) attn_bwd_prep_kernel(const floa
     }
     for (int e = threadIdx.x; e < d; e += kSmallThreads) gs[e] = G[i * d + e];
     __syncthreads();
-    row_dots(gs, WV, C, d, [&](int c, float s) {
+    row_dots_serial(gs, WV, C, d, tile, [&](int c, float s) {
         dO[i * C + c] = s;
         dO_bf[i * C + c] = __float2bfloat16_rn(s);
         part[c] = s * O[i * C + c];
     });
     __syncthreads();
-    if (threadIdx.x < 32) {
+    const int w = threadIdx.x >> 5;
+    if (w < C / 32) {
+        const float s = warp_sum(part[threadIdx.x]);
+        if ((threadIdx.x & 31) == 0) red[w] = s;
+    }
+    __syncthreads();
+    if (threadIdx.x == 0) {
         float s = 0.0f;
-        for (int c = threadIdx.x; c < C; c += 32) s += part[c];
-        s = warp_sum(s);
-        if (threadIdx.x == 0) Dq[i] = s;
+        for (int k = 0; k < C / 32; ++k) s += red[k];
+        Dq[i] = s;
     }
 }
 
