@@ -233,7 +233,7 @@ __device__ __forceinline__ void group_transpose_sum16(float v[16], int lane)
 // gradient is summed by the whole warp, lanes across channels (NG = 1).
 template <int KMAX, int DT, int CH, bool SAVED, bool LP, int TH, bool NW = false>
 __device__ __forceinline__ void bwd_tile(const FrameParams &fp, const BwdArgs &a, Pipe &P, HitLists *hits,
-                                         int &s_maxlast, uint32_t tile)
+                                         int &s_maxlast, float4 *feat_stage, uint32_t tile)
 {
     constexpr int PW = pixel_warps(TH);
     constexpr int kSlots = LP ? 16 : 12;
@@ -391,12 +391,19 @@ __device__ __forceinline__ void bwd_tile(const FrameParams &fp, const BwdArgs &a
         __syncthreads();
     }
     const int maxlast = s_maxlast;
-    if (producer) {
-        pipe_produce<LP, PW>(P, a.vals, list0, maxlast, true, a.records, tileX, tileY, a.status, kSiteRenderBwdB,
-                             rec_lo, rec_hi);
-        return;
-    }
-    pipe_prefill<LP, PW>(P, wid, a.vals, list0, maxlast, true, a.records, tileX, tileY, a.status, rec_lo, rec_hi);
+    auto stage = [&](const auto &extra) {
+        if (producer)
+            pipe_produce<LP, PW>(P, a.vals, list0, maxlast, true, a.records, tileX, tileY, a.status, kSiteRenderBwdB,
+                                 rec_lo, rec_hi, extra);
+        else
+            pipe_prefill<LP, PW>(P, wid, a.vals, list0, maxlast, true, a.records, tileX, tileY, a.status, rec_lo,
+                                 rec_hi, extra);
+    };
+    if constexpr (NW)
+        stage(StageFeat<DT, 16>{a.g_F ? a.feat : nullptr, 16, 0, a.wide, rec_lo, feat_stage});
+    else
+        stage(NoExtra());
+    if (producer) return;
     if constexpr (ext_feat) sel_saved.init(a, pix, K, inside);
     // entries at or beyond every lane's last composited surfel are skipped by
     // the group (the warp when it walks one list)
@@ -477,7 +484,7 @@ __device__ __forceinline__ void bwd_tile(const FrameParams &fp, const BwdArgs &a
                         } else if (NW && a.g_F && a.feat) {
                             sel = true;
                             float f[16];
-                            load_feat<DT, 16>(a.feat, sid, 16, 0, f, a.wide);
+                            staged_feat<16>(feat_stage, st, j, f);
                             if (a.fscale) {
 #pragma unroll
                                 for (int c = 0; c < 16; ++c) dot = fmaf(gfr[c] * __ldg(a.fscale + c), f[c], dot);
@@ -814,13 +821,14 @@ __global__ void __launch_bounds__(pipe_threads(TH), OCC)
 {
     __shared__ __align__(128) Pipe P;
     __shared__ HitLists hits[pixel_warps(TH)];
+    extern __shared__ __align__(16) float4 feat_stage[]; // NW: feat_stage_bytes(16)
     __shared__ int s_maxlast;
     __shared__ uint32_t s_next;
     uint32_t i = blockIdx.x;
     while (true) {
         const uint32_t tile = a.ranges[2 * fp.n_tiles_total + i];
         if (PSI_CHECK(tile < fp.n_tiles_total, kChkTile, a.status))
-            bwd_tile<KMAX, DT, CH, SAVED, LP, TH, NW>(fp, a, P, hits, s_maxlast, tile);
+            bwd_tile<KMAX, DT, CH, SAVED, LP, TH, NW>(fp, a, P, hits, s_maxlast, feat_stage, tile);
         if (!a.work) break;
         __syncthreads();
         if (threadIdx.x == 0) {
@@ -959,16 +967,20 @@ cudaError_t launch_kcslo(const FrameParams &fp, const FeatView &f, const BwdArgs
     if (a.work) grid = persistent_grid(fp.n_tiles_total, OCC);
     constexpr int nt = pipe_threads(TH);
     if constexpr (KMAX == 0 && CH == 16) {
-        // dense 16-channel tables: the register-held g_F row
+        // dense 16-channel tables: the register-held g_F row, the table's rows staged with the records
         if (f.data && f.dim == 16) {
+            auto launch = [&](auto kernel) {
+                constexpr size_t dyn = feat_stage_bytes(16);
+                const cudaError_t e = cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, static_cast<int>(dyn));
+                if (e != cudaSuccess) return e;
+                kernel<<<grid, nt, dyn, st>>>(fp, a);
+                return cudaGetLastError();
+            };
             switch (f.dtype) {
-            case PSI_BF16: render_bwd_kernel<0, PSI_BF16, 16, SAVED, LP, OCC, TH, true><<<grid, nt, 0, st>>>(fp, a); break;
-            case PSI_FP8_E4M3:
-                render_bwd_kernel<0, PSI_FP8_E4M3, 16, SAVED, LP, OCC, TH, true><<<grid, nt, 0, st>>>(fp, a);
-                break;
-            default: render_bwd_kernel<0, PSI_F32, 16, SAVED, LP, OCC, TH, true><<<grid, nt, 0, st>>>(fp, a); break;
+            case PSI_BF16: return launch(render_bwd_kernel<0, PSI_BF16, 16, SAVED, LP, OCC, TH, true>);
+            case PSI_FP8_E4M3: return launch(render_bwd_kernel<0, PSI_FP8_E4M3, 16, SAVED, LP, OCC, TH, true>);
+            default: return launch(render_bwd_kernel<0, PSI_F32, 16, SAVED, LP, OCC, TH, true>);
             }
-            return cudaGetLastError();
         }
     }
     switch (f.data ? f.dtype : PSI_F32) {

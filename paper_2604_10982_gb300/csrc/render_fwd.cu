@@ -275,12 +275,20 @@ __device__ __forceinline__ void fwd_tile(const FrameParams &fp, const FwdArgs &a
     const int vw = wid + (oy ? pixel_warps(16) / 2 : 0); // warp of the 16x16 tile this warp plays
     if (tid == 0) pipe_init(P, PW, wlimit);
     __syncthreads();
-    if (wid == PW) {
-        pipe_produce<LP, PW>(P, a.vals, list0, n, false, a.records, tx * kTile, ty * TH - oy, a.status, kSiteRenderFwd,
-                             rec_lo, rec_hi);
-        return;
-    }
-    pipe_prefill<LP, PW>(P, wid, a.vals, list0, n, false, a.records, tx * kTile, ty * TH - oy, a.status, rec_lo, rec_hi);
+    auto stage = [&](const auto &extra) {
+        if (wid == PW)
+            pipe_produce<LP, PW>(P, a.vals, list0, n, false, a.records, tx * kTile, ty * TH - oy, a.status,
+                                 kSiteRenderFwd, rec_lo, rec_hi, extra);
+        else
+            pipe_prefill<LP, PW>(P, wid, a.vals, list0, n, false, a.records, tx * kTile, ty * TH - oy, a.status, rec_lo,
+                                 rec_hi, extra);
+    };
+    // dense features: this pass's channels are staged with the records
+    if constexpr (KMAX == 0)
+        stage(StageFeat<DT, CH>{a.feat, a.D, a.c0, a.wide, rec_lo, entries});
+    else
+        stage(NoExtra());
+    if (wid == PW) return;
 
     int lxi, lyi;
     pixel_of_thread(vw * 32 + lane, lxi, lyi);
@@ -336,7 +344,7 @@ __device__ __forceinline__ void fwd_tile(const FrameParams &fp, const FwdArgs &a
                 if constexpr (KMAX == 0) {
                     if (a.feat) {
                         float f[CH];
-                        load_feat<DT, CH>(a.feat, static_cast<int64_t>(P.val[st][j]) - surf0, a.D, a.c0, f, a.wide);
+                        staged_feat<CH>(entries, st, j, f);
 #pragma unroll
                         for (int c = 0; c < CH; ++c) facc[c] = __fmaf_rn(w, f[c], facc[c]);
                     }
@@ -433,7 +441,7 @@ __global__ void __launch_bounds__(pipe_threads(TH), OCC)
     __shared__ __align__(128) PipeT<(KMAX > 8 ? 3 : 4)> P;
     __shared__ HitLists hits[pixel_warps(TH)];
     __shared__ uint32_t s_next;
-    extern __shared__ __align__(16) float4 entries[]; // topk_entries(K) per pixel warp
+    extern __shared__ __align__(16) float4 entries[]; // K > 0: topk_entries(K) per pixel warp; dense: feature stages
     uint32_t i = blockIdx.x;
     while (true) {
         const uint32_t tile = a.ranges[2 * fp.n_tiles_total + i];
@@ -463,9 +471,10 @@ cudaError_t launch_one(const FrameParams &fp, const FwdArgs &a, cudaStream_t st)
 {
     const auto kernel = render_fwd_kernel<KMAX, DT, CH, LP, OCC, TH>;
     const unsigned grid = a.work ? persistent_grid(fp.n_tiles_total, OCC) : fp.n_tiles_total;
-    const size_t dyn = KMAX > 0 ? static_cast<size_t>(pixel_warps(TH)) * topk_entries(fp.top_k) * sizeof(float4) : 0;
-    if (KMAX > 0) {
-        // the sets and the stages together pass 48 KB
+    const size_t dyn = KMAX > 0 ? static_cast<size_t>(pixel_warps(TH)) * topk_entries(fp.top_k) * sizeof(float4)
+                                : (a.feat ? feat_stage_bytes(CH) : 0);
+    if (dyn > 0) {
+        // the sets or features and the record stages together pass 48 KB
         const cudaError_t e = cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, static_cast<int>(dyn));
         if (e != cudaSuccess) return e;
     }
