@@ -128,9 +128,9 @@ __device__ __forceinline__ void load_sorted_set(const FrameParams &fp, const Fea
     }
 }
 
-// NCH: 16-byte channel chunks per lane (1: D <= 128, 2: D <= 256).
-template <int KMAX, int DT, int NCH>
-__global__ void __launch_bounds__(256, (KMAX <= 8 && NCH == 1) ? 4 : 1) feat_bwd_kernel(const __grid_constant__ FrameParams fp, FeatBwdArgs a)
+// 128 < D <= 256: two 16-byte channel chunks per lane.
+template <int KMAX, int DT>
+__global__ void __launch_bounds__(256, 1) feat_bwd_kernel(const __grid_constant__ FrameParams fp, FeatBwdArgs a)
 {
     const int tid = threadIdx.x, lane = tid & 31;
     const uint32_t tile = blockIdx.x;
@@ -154,7 +154,7 @@ __global__ void __launch_bounds__(256, (KMAX <= 8 && NCH == 1) ? 4 : 1) feat_bwd
 
     // lane l owns channels [4l, 4l + 4) and [4l + 128, 4l + 132) (D <= 256)
     const int nv = a.D >> 2;
-    const bool c0on = lane < nv, c1on = NCH > 1 && lane + 32 < nv;
+    const bool c0on = lane < nv, c1on = lane + 32 < nv;
     float4 sc0 = make_float4(1.f, 1.f, 1.f, 1.f), sc1 = sc0;
     if (a.fscale) {
         const float *p = a.fscale + 4 * lane; // the scale array has no alignment beyond 4 bytes
@@ -359,14 +359,14 @@ __global__ void __launch_bounds__(256, 2) feat_bwd_reg_kernel(const __grid_const
     }
 }
 
-template <int KMAX, int NCH>
-cudaError_t launch_kn(const FrameParams &fp, const FeatView &f, const FeatBwdArgs &a, cudaStream_t st)
+template <int KMAX>
+cudaError_t launch_wide(const FrameParams &fp, const FeatView &f, const FeatBwdArgs &a, cudaStream_t st)
 {
     const unsigned grid = static_cast<unsigned>(fp.n_tiles_total);
     switch (f.dtype) {
-    case PSI_BF16: feat_bwd_kernel<KMAX, PSI_BF16, NCH><<<grid, 16 * fp.tile_h, 0, st>>>(fp, a); break;
-    case PSI_FP8_E4M3: feat_bwd_kernel<KMAX, PSI_FP8_E4M3, NCH><<<grid, 16 * fp.tile_h, 0, st>>>(fp, a); break;
-    default: feat_bwd_kernel<KMAX, PSI_F32, NCH><<<grid, 16 * fp.tile_h, 0, st>>>(fp, a); break;
+    case PSI_BF16: feat_bwd_kernel<KMAX, PSI_BF16><<<grid, 16 * fp.tile_h, 0, st>>>(fp, a); break;
+    case PSI_FP8_E4M3: feat_bwd_kernel<KMAX, PSI_FP8_E4M3><<<grid, 16 * fp.tile_h, 0, st>>>(fp, a); break;
+    default: feat_bwd_kernel<KMAX, PSI_F32><<<grid, 16 * fp.tile_h, 0, st>>>(fp, a); break;
     }
     return cudaGetLastError();
 }
@@ -387,7 +387,7 @@ cudaError_t launch_reg(const FrameParams &fp, const FeatBwdArgs &a, cudaStream_t
 template <int KMAX>
 cudaError_t launch_k(const FrameParams &fp, const FeatView &f, const FeatBwdArgs &a, cudaStream_t st)
 {
-    if (f.dim > 128) return launch_kn<KMAX, 2>(fp, f, a, st);
+    if (f.dim > 128) return launch_wide<KMAX>(fp, f, a, st);
     switch (f.dtype) {
     case PSI_BF16: return launch_reg<KMAX, PSI_BF16>(fp, a, st);
     case PSI_FP8_E4M3: return launch_reg<KMAX, PSI_FP8_E4M3>(fp, a, st);
