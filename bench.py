@@ -397,7 +397,8 @@ def run_psi(args):
         tuned = {"tile": f"16x{int(opts.tile_h)}", "frame_ms_per_tile_height": tile_ms,
                  "forward": {"ms_per_shape": [round(x, 4) for x in tr["fwd"][0]], "shape": tr["fwd"][1]},
                  "adjoint": {"ms_per_shape": [round(x, 4) for x in tr["bwd"][0]], "shape": tr["bwd"][1]},
-                 "shapes": "bit 0: the other CTAs-per-SM build (K<=8: forward 3->4, adjoint from saved state 4->3, else 2->1); "
+                 "shapes": "bit 0: the other CTAs-per-SM build (K<=8: forward 3->4, adjoint from saved state 4->3, "
+                           "K>8 3->4; forward K 9..16: 3->2; else 2->1); "
                            "bit 1: dense 16-channel passes; bit 2: persistent launch (tile counter); bit 3: adjoint "
                            "walk with two pixels per lane instead of one (saved state, K>0); -1: shape does not apply; "
                            "tile height and shapes timed on frame 0 before the graphs are captured"}
