@@ -185,7 +185,9 @@ int psi_status_fetch(psi_ctx *ctx, psi_stream stream, int32_t *status_out, int64
  * are released. psi_ctx_set_wait_limit_ns sets the limit for kernels launched
  * after it returns (0 restores 1 s; at most PSI_WAIT_LIMIT_MAX_NS, else
  * PSI_ERR_INVALID_ARG). A limit shorter than a kernel's normal waits makes
- * its outputs invalid: it exists to exercise the give-up path. Synchronous
+ * its outputs invalid: it exists to exercise the give-up path (compositing and
+ * intersect take a limit below 1024 ns, the timer's coarsest step, as run out at the
+ * first poll that fails). Synchronous
  * copy to the device: not inside a stream capture. */
 #define PSI_WAIT_LIMIT_MAX_NS 10000000000ull
 int psi_ctx_set_wait_limit_ns(psi_ctx *ctx, uint64_t ns);
@@ -247,7 +249,9 @@ int psi_project_surfels(psi_ctx *ctx, const psi_surfels *s, const psi_camera *ca
  *  keys, vals:  [capacity]; d_num_pairs: device int64 receiving the pair count
  *  workspace:   psi_intersect_workspace_size(n_views*N) bytes
  * If the count exceeds capacity, pairs beyond it are dropped, *d_num_pairs is
- * clamped to capacity and PSI_ERR_CAPACITY is raised on the device. */
+ * clamped to capacity and PSI_ERR_CAPACITY is raised on the device. If a wait
+ * of the prefix sums gives up (PSI_ERR_TIMEOUT), *d_num_pairs is 0: the stages
+ * queued behind it see an empty frame. */
 int psi_intersect_tiles(psi_ctx *ctx, const psi_camera *cams, int n_views, const psi_render_opts *o,
                         int64_t n_surfels, const void *bin_records, const uint32_t *tiles_touched, uint64_t *keys,
                         uint32_t *vals, int64_t capacity, int64_t *d_num_pairs, void *workspace,

@@ -117,6 +117,19 @@ __device__ __forceinline__ unsigned long long global_ns()
     return t;
 }
 
+// %globaltimer may advance in steps of a microsecond: a limit below one step
+// has run out at the first poll that fails.
+constexpr unsigned long long kTimerTickNs = 1024;
+
+// After a failed poll: whether the wait that started at t0 (0 before its first
+// failed poll) has lasted longer than `limit`.
+__device__ __forceinline__ bool wait_expired(unsigned long long &t0, unsigned long long limit)
+{
+    const unsigned long long now = global_ns();
+    if (t0 == 0) t0 = now;
+    return limit < kTimerTickNs || now - t0 > limit;
+}
+
 __device__ __forceinline__ uint32_t smem_u32(const void *p)
 {
     return static_cast<uint32_t>(__cvta_generic_to_shared(p));

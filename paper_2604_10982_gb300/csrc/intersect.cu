@@ -10,7 +10,7 @@
 // One kernel: a block takes the next 1024 records (a ticket, so that every
 // predecessor is already running), sums their tile counts, learns where its
 // pairs start from its predecessors' published sums (decoupled look-back, a
-// bounded wait per word), gathers its visible records -- half of a street's
+// bounded wait per word; if one runs out the frame has no pairs), gathers its visible records -- half of a street's
 // are culled -- and emits them one per thread. The counts are read once and no
 // offsets are stored; up to 3072 pairs of a block are assembled in shared
 // memory, so that its stores are contiguous (a thread writing its record's pairs
@@ -32,37 +32,46 @@ constexpr int kRecords = kThreads * kItems;  // records per block
 constexpr int kStage = 3072;                 // pairs assembled in shared memory
 constexpr unsigned long long kOneRecord = 1ull << 48; // a visible record in the sums of pairs
 
-// look-back word of a block: flag in bits 62-63, the pair count below
+// look-back word of a block: flag in bits 62-63, bit 61 set if the sum is not
+// known because a wait gave up, the pair count below
 constexpr unsigned long long kFlagAgg = 1ull << 62;  // the block's own count
 constexpr unsigned long long kFlagIncl = 2ull << 62; // the count of all blocks up to this one
-constexpr unsigned long long kValueMask = (1ull << 62) - 1ull;
+constexpr unsigned long long kFlags = 3ull << 62;
+constexpr unsigned long long kPoison = 1ull << 61;
+constexpr unsigned long long kValueMask = kPoison - 1ull;
 
 // Pairs of all blocks before `part` (one warp; every lane gets the sum): the
-// predecessors' words, 32 at a time, back to the first inclusive one.
-__device__ __forceinline__ unsigned long long look_back(const unsigned long long *words, int64_t part, DevStatus *status)
+// predecessors' words, 32 at a time, back to the first inclusive one. `ok` is
+// false, and the sum meaningless, if a wait ran out here or at a predecessor.
+__device__ __forceinline__ unsigned long long look_back(const unsigned long long *words, int64_t part,
+                                                        DevStatus *status, bool &ok)
 {
     const int lane = threadIdx.x & 31;
     const unsigned long long limit = wait_limit(status);
     unsigned long long excl = 0;
+    ok = true;
     for (int64_t q = part - 1; q >= 0; q -= 32) {
         const int64_t idx = q - lane;
         unsigned long long w = kFlagIncl; // before the first block: nothing
         unsigned long long t0 = 0;
         while (true) {
             if (idx >= 0) w = *reinterpret_cast<const volatile unsigned long long *>(words + idx);
-            if (__all_sync(0xffffffffu, (w & ~kValueMask) != 0)) break;
-            const unsigned long long now = global_ns();
-            if (t0 == 0) t0 = now;
-            if (__any_sync(0xffffffffu, now - t0 > limit)) {
+            if (__all_sync(0xffffffffu, (w & kFlags) != 0)) break;
+            if (__any_sync(0xffffffffu, wait_expired(t0, limit))) {
                 if (lane == 0 && status) {
                     atomicCAS(&status->wait_site, 0, kSiteIntersect);
                     raise_status(status, PSI_ERR_TIMEOUT);
                 }
-                return excl;
+                ok = false;
+                return 0;
             }
         }
         const uint32_t incl = __ballot_sync(0xffffffffu, (w & kFlagIncl) != 0);
         const int first = incl ? __ffs(incl) - 1 : 31;
+        if (__any_sync(0xffffffffu, lane <= first && (w & kPoison))) {
+            ok = false;
+            return 0;
+        }
         unsigned long long v = lane <= first ? (w & kValueMask) : 0ull;
 #pragma unroll
         for (int o = 16; o > 0; o >>= 1) v += __shfl_xor_sync(0xffffffffu, v, o);
@@ -78,7 +87,7 @@ __global__ void __launch_bounds__(kThreads) intersect_kernel(const __grid_consta
                                                              uint64_t *__restrict__ keys, uint32_t *__restrict__ vals,
                                                              int64_t capacity, int64_t *__restrict__ d_num_pairs,
                                                              unsigned long long *words, unsigned int *ticket,
-                                                             DevStatus *status)
+                                                             unsigned long long *finished, DevStatus *status)
 {
     __shared__ uint64_t s_keys[kStage];
     __shared__ uint32_t s_vals[kStage];
@@ -86,6 +95,7 @@ __global__ void __launch_bounds__(kThreads) intersect_kernel(const __grid_consta
     __shared__ uint16_t s_rec[kRecords];
     __shared__ unsigned long long warp_sum[kWarps];
     __shared__ unsigned long long s_base;
+    __shared__ bool s_ok;
     __shared__ unsigned int s_part;
     const int tid = threadIdx.x, lane = tid & 31, wid = tid >> 5;
     if (tid == 0) s_part = atomicAdd(ticket, 1u);
@@ -132,27 +142,39 @@ __global__ void __launch_bounds__(kThreads) intersect_kernel(const __grid_consta
     if (wid == 0) {
         volatile unsigned long long *my = words + part;
         unsigned long long excl = 0;
+        bool ok = true;
         if (part > 0) {
             if (lane == 0) *my = kFlagAgg | all;
-            excl = look_back(words, part, status);
+            excl = look_back(words, part, status, ok);
         }
         if (lane == 0) {
-            *my = kFlagIncl | (excl + all);
+            *my = kFlagIncl | (ok ? excl + all : kPoison);
             s_base = excl;
+            s_ok = ok;
         }
     }
     __syncthreads();
     const unsigned long long base = s_base;
     const unsigned long long cap = static_cast<unsigned long long>(capacity);
-    if (rec0 + kRecords >= total && tid == 0) {
-        // the last block knows the frame's count
-        if (base + all > cap) {
-            raise_status(status, PSI_ERR_CAPACITY);
-            atomicMax(&status->required_pairs, base + all);
+    if (tid == kThreads - 1) {
+        // The block that finishes last (not the frame's last block: one before
+        // it may still give up) knows whether every block has its place, and
+        // the frame's count: without it the list would have holes, so there is none.
+        __threadfence();
+        const unsigned long long old = atomicAdd(finished, s_ok ? 1ull : (1ull << 32) + 1ull);
+        if (static_cast<uint32_t>(old) == gridDim.x - 1) {
+            __threadfence();
+            const bool whole = s_ok && (old >> 32) == 0;
+            const unsigned long long w = *reinterpret_cast<const volatile unsigned long long *>(words + gridDim.x - 1);
+            const unsigned long long pairs = whole ? w & kValueMask : 0ull;
+            if (pairs > cap) {
+                raise_status(status, PSI_ERR_CAPACITY);
+                atomicMax(&status->required_pairs, pairs);
+            }
+            *d_num_pairs = static_cast<int64_t>(pairs < cap ? pairs : cap);
         }
-        *d_num_pairs = static_cast<int64_t>(base + all < cap ? base + all : cap);
     }
-    if (base >= cap) return;
+    if (!s_ok || base >= cap) return;
 
     // one visible record per thread
     const bool staged = all <= kStage;
@@ -198,10 +220,10 @@ int64_t blocks_of(int64_t n_records) { return (n_records + kRecords - 1) / kReco
 
 } // namespace
 
-// the look-back words and the ticket
+// the look-back words, the ticket and the finished blocks' count
 size_t intersect_workspace_bytes(int64_t n_records)
 {
-    return align_up(static_cast<size_t>(blocks_of(std::max<int64_t>(n_records, 1))) * 8 + 8, 256);
+    return align_up(static_cast<size_t>(blocks_of(std::max<int64_t>(n_records, 1))) * 8 + 16, 256);
 }
 
 cudaError_t launch_intersect(const FrameParams &fp, const float4 *bin_records, const uint32_t *tiles_touched,
@@ -213,10 +235,10 @@ cudaError_t launch_intersect(const FrameParams &fp, const float4 *bin_records, c
     const int64_t nb = blocks_of(R);
     auto *words = static_cast<unsigned long long *>(ws);
     auto *ticket = reinterpret_cast<unsigned int *>(words + nb);
-    cudaError_t e = cudaMemsetAsync(ws, 0, static_cast<size_t>(nb) * 8 + 8, st);
+    cudaError_t e = cudaMemsetAsync(ws, 0, static_cast<size_t>(nb) * 8 + 16, st);
     if (e != cudaSuccess) return e;
     intersect_kernel<<<static_cast<unsigned>(nb), kThreads, 0, st>>>(fp, bin_records, tiles_touched, keys, vals, capacity,
-                                                                    d_num_pairs, words, ticket, status);
+                                                                    d_num_pairs, words, ticket, words + nb + 1, status);
     return cudaGetLastError();
 }
 

@@ -205,7 +205,6 @@ constexpr int kPixelWarps = pixel_warps(16);
 constexpr int kPipeThreads = pipe_threads(16);
 
 constexpr int kLeft = 0x7fffffff;  // released[w] of a warp that left the walk
-constexpr unsigned long long kTimerTickNs = 1024; // %globaltimer may advance in steps of a microsecond
 constexpr uint32_t kSuspendNs = 20000; // longest hardware suspension per poll of a wait
 
 // NS stages: 4, or 3 where a fourth costs a resident CTA (with two of them
