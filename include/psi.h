@@ -185,9 +185,9 @@ int psi_status_fetch(psi_ctx *ctx, psi_stream stream, int32_t *status_out, int64
  * are released. psi_ctx_set_wait_limit_ns sets the limit for kernels launched
  * after it returns (0 restores 1 s; at most PSI_WAIT_LIMIT_MAX_NS, else
  * PSI_ERR_INVALID_ARG). A limit shorter than a kernel's normal waits makes
- * its outputs invalid: it exists to exercise the give-up path (compositing and
- * intersect take a limit below 1024 ns, the timer's coarsest step, as run out at the
- * first poll that fails). Synchronous
+ * its outputs invalid: it exists to exercise the give-up path (compositing,
+ * intersect and sort take a limit below 1024 ns, the timer's coarsest step, as run out
+ * at the first poll that fails). Synchronous
  * copy to the device: not inside a stream capture. */
 #define PSI_WAIT_LIMIT_MAX_NS 10000000000ull
 int psi_ctx_set_wait_limit_ns(psi_ctx *ctx, uint64_t ns);
@@ -268,7 +268,9 @@ int psi_intersect_tiles(psi_ctx *ctx, const psi_camera *cams, int n_views, const
  * Pass begin_bit=0, end_bit=32+ceil(log2(n_tiles_total)) for the full order.
  * If *d_num_pairs exceeds capacity, only the first capacity pairs are sorted
  * and ranged, and PSI_ERR_CAPACITY (detail: *d_num_pairs) is raised on the
- * device; nothing is read or written past capacity.
+ * device; nothing is read or written past capacity. If a wait of the sort
+ * gives up (PSI_ERR_TIMEOUT), every tile's range is empty and keys / vals hold
+ * an unspecified arrangement.
  *  workspace: psi_sort_workspace_size(capacity) bytes. */
 int psi_sort_keys(psi_ctx *ctx, uint64_t *keys, uint32_t *vals, const int64_t *d_num_pairs, int64_t capacity,
                   int begin_bit, int end_bit, uint32_t *tile_ranges, int64_t n_tiles_total, void *workspace,

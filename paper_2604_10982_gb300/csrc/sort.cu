@@ -8,7 +8,8 @@
 // in launch order, so every predecessor is already running), ranks its items
 // stably (warp match on the digit, per-warp running counters, prefix over
 // warps), publishes its per-digit counts, reads its predecessors' published
-// counts back to the first inclusive prefix (a bounded wait on each flag) to
+// counts back to the first inclusive prefix (a bounded wait on each flag; if
+// one runs out, nothing more is moved and every tile's range stays empty) to
 // learn where its run of every digit starts, and writes its items out through
 // shared memory so that runs of one digit leave the block as contiguous,
 // coalesced stores. The number of passes is made even so the result ends in
@@ -101,6 +102,9 @@ constexpr unsigned long long kFlagAgg = 1ull << 62;  // this partition's own cou
 constexpr unsigned long long kFlagIncl = 2ull << 62; // count of all partitions up to this one
 constexpr unsigned long long kTagMask = 15ull << 58;
 constexpr unsigned long long kValueMask = (1ull << 58) - 1ull;
+// in the partition counters of a pass and all later ones: a wait of the pass
+// ran out (a partition taken from such a counter lies past any pair count)
+constexpr unsigned int kGaveUp = 1u << 31;
 __device__ __forceinline__ unsigned long long pass_tag(int ps) { return static_cast<unsigned long long>(ps + 1) << 58; }
 
 struct ScatterSmem {
@@ -130,7 +134,9 @@ __global__ void __launch_bounds__(kThreads) onesweep_kernel(const uint64_t *__re
     const int64_t part = s_part;
     const int64_t n = clamped_count(d_n, cap);
     const int64_t blk0 = part * kTile;
-    if (blk0 >= n) return; // partitions are handed out in order: no valid one waits for this
+    // past the end: partitions are handed out in order, no valid one waits for
+    // this; or a wait gave up and this pass's input may have holes
+    if (blk0 >= n) return;
     const uint64_t mask = (bits >= 64) ? ~0ull : ((1ull << bits) - 1ull);
     for (int k = threadIdx.x; k < kWarps * kBins; k += kThreads) (&S.warp_cnt[0][0])[k] = 0;
     __syncthreads();
@@ -178,6 +184,7 @@ __global__ void __launch_bounds__(kThreads) onesweep_kernel(const uint64_t *__re
     // publish this partition's count of digit d, then read the predecessors'
     // back to the first inclusive prefix: the block's run of digit d starts at
     // digit_base[d] + (items of digit d in all earlier partitions)
+    bool lost = false; // a wait ran out here or in another block
     {
         const int d = threadIdx.x;
         volatile unsigned long long *row = status_words + part * kBins;
@@ -189,16 +196,21 @@ __global__ void __launch_bounds__(kThreads) onesweep_kernel(const uint64_t *__re
             row[d] = kFlagAgg | tag | cnt;
             const unsigned long long limit = wait_limit(status);
             unsigned long long t0 = 0;
+            unsigned int polls = 0;
             for (int64_t q = part - 1; q >= 0;) {
                 const unsigned long long w = reinterpret_cast<volatile unsigned long long *>(status_words)[q * kBins + d];
                 if ((w & (kFlagAgg | kFlagIncl)) == 0 || (w & kTagMask) != tag) {
-                    const unsigned long long now = global_ns();
-                    if (t0 == 0) t0 = now;
-                    else if (now - t0 > limit) {
+                    // a predecessor that gave up publishes nothing: look for that now and then
+                    if ((++polls & 63u) == 0)
+                        lost = (*reinterpret_cast<volatile unsigned int *>(part_counter) & kGaveUp) != 0;
+                    if (lost) break;
+                    if (wait_expired(t0, limit)) {
                         if (status) {
                             atomicCAS(&status->wait_site, 0, kSiteSort);
                             raise_status(status, PSI_ERR_TIMEOUT);
                         }
+                        for (int p = ps; p < kMaxPasses; ++p) atomicOr(part_counter + (p - ps), kGaveUp);
+                        lost = true;
                         break;
                     }
                     continue;
@@ -208,7 +220,7 @@ __global__ void __launch_bounds__(kThreads) onesweep_kernel(const uint64_t *__re
                 if (w & kFlagIncl) break;
                 --q;
             }
-            row[d] = kFlagIncl | tag | (excl + cnt);
+            if (!lost) row[d] = kFlagIncl | tag | (excl + cnt);
         }
         S.digit_base[d] = static_cast<unsigned long long>(digit_base[d]) + excl;
     }
@@ -220,7 +232,7 @@ __global__ void __launch_bounds__(kThreads) onesweep_kernel(const uint64_t *__re
         if (lane >= o) inc += t;
     }
     if (lane == 31) S.warp_tot[wid] = inc;
-    __syncthreads();
+    if (__syncthreads_or(lost)) return;
     if (wid == 0) {
         const uint32_t t = lane < kWarps ? S.warp_tot[lane] : 0u;
         uint32_t ti = t;
@@ -258,11 +270,13 @@ __global__ void __launch_bounds__(kThreads) onesweep_kernel(const uint64_t *__re
 
 __global__ void __launch_bounds__(256) ranges_kernel(const uint64_t *__restrict__ keys, const int64_t *__restrict__ d_n,
                                                      int64_t cap, uint32_t *__restrict__ ranges, int64_t n_tiles,
+                                                     const unsigned int *__restrict__ last_counter,
                                                      DevStatus *status)
 {
+    const bool gave_up = (*last_counter & kGaveUp) != 0; // the keys are not sorted: every range stays empty
     const int64_t n = clamped_count(d_n, cap);
     const int64_t i = static_cast<int64_t>(blockIdx.x) * blockDim.x + threadIdx.x;
-    if (i >= n) return;
+    if (i >= n || gave_up) return;
     const uint64_t t = keys[i] >> 32;
     if (t >= static_cast<uint64_t>(n_tiles)) {
         raise_status(status, PSI_ERR_INVALID_ARG);
@@ -545,7 +559,8 @@ cudaError_t launch_sort(uint64_t *keys, uint32_t *vals, const int64_t *d_num_pai
         e = cudaMemsetAsync(tile_ranges, 0, static_cast<size_t>(n_tiles_total) * 8, st);
         if (e != cudaSuccess) return e;
         ranges_kernel<<<static_cast<unsigned>((cap + 255) / 256), 256, 0, st>>>(keys, d_num_pairs, cap, tile_ranges,
-                                                                               n_tiles_total, status);
+                                                                               n_tiles_total, counters + kMaxPasses - 1,
+                                                                               status);
         tile_order_kernel<<<1, 1024, 0, st>>>(tile_ranges, n_tiles_total, tile_ranges + 2 * n_tiles_total);
     }
     return cudaGetLastError();

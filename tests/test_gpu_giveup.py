@@ -80,3 +80,45 @@ def test_intersect_giveup_leaves_no_pairs(ctx):
     assert int(r.num_pairs.item()) == pairs and _intact(keys_b, vals_b, ws_b)
     for a, b in zip(outs(), clean):
         assert torch.equal(a, b)
+
+
+@pytest.mark.parametrize("n,passes_bits", [(300_000, 45), (2_000_000, 61)])
+def test_sort_giveup_leaves_empty_lists(ctx, n, passes_bits):
+    """74 and 489 partitions, 6 and 8 passes. A poll fails as soon as a partition
+    is ahead of its predecessor."""
+    from paper_2604_10982_gb300 import psi
+    n_tiles, capacity = 1500, n + 5
+    rng = np.random.default_rng(n)
+    keys = (rng.integers(0, n_tiles, n).astype(np.uint64) << np.uint64(32)) | rng.integers(0, 2**31, n).astype(np.uint64)
+    pad = np.full(capacity - n, 7, np.uint64)
+    k0 = torch.from_numpy(np.concatenate([keys, pad]).view(np.int64)).cuda()
+    v0 = torch.arange(capacity, dtype=torch.int32, device="cuda")
+    keys_b, k = _guarded(capacity, torch.int64)
+    vals_b, v = _guarded(capacity, torch.int32)
+    rg_b, ranges = _guarded(3 * n_tiles, torch.int32)
+    ws_b, ws = _guarded(psi.sort_workspace_size(capacity), torch.uint8)
+    num = torch.tensor([n], dtype=torch.int64, device="cuda")
+
+    def sort():
+        k.copy_(k0)
+        v.copy_(v0)
+        psi.psi_sort_keys(ctx, k, v, num, capacity, 0, passes_bits, ranges, n_tiles, ws)
+        return ctx.status_fetch()
+
+    psi.psi_ctx_set_wait_limit_ns(ctx, 1)
+    for _ in range(TRIES):
+        st = sort()
+        if st[0]:
+            break
+    assert st == (psi.PSI_ERR_TIMEOUT, 8)
+    assert torch.count_nonzero(ranges[:2 * n_tiles]).item() == 0
+    assert torch.equal(ranges[2 * n_tiles:].sort()[0], torch.arange(n_tiles, dtype=torch.int32, device="cuda"))
+    assert _intact(keys_b, vals_b, rg_b, ws_b)
+    assert torch.equal(k[n:], k0[n:]) and torch.equal(v[n:], v0[n:])
+
+    psi.psi_ctx_set_wait_limit_ns(ctx, 0)
+    assert sort() == (0, 0)
+    order = np.argsort(keys, kind="stable")
+    assert np.array_equal(k.cpu().numpy().view(np.uint64)[:n], keys[order])
+    assert np.array_equal(v.cpu().numpy()[:n], order.astype(np.int32))
+    assert _intact(keys_b, vals_b, rg_b, ws_b)
