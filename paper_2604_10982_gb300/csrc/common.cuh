@@ -341,6 +341,16 @@ cudaError_t launch_labels(const void *F, int64_t n, int D, const float *centres,
 cudaError_t launch_decode(const void *F, int64_t n_pix, int D, const void *Q, int n_q, const float *T, int32_t *ids,
                           void *logits, DevStatus *status, cudaStream_t st, const char **why);
 
+// Opts a kernel in to `bytes` of dynamic shared memory. The limit is one value
+// per kernel and device, shared by every host thread, so a kernel always gets
+// the same one -- the most any call of it uses, not this call's size, which
+// another thread's smaller call could undercut before the launch.
+template <class Kernel>
+inline cudaError_t allow_dynamic_smem(Kernel kernel, size_t bytes)
+{
+    return cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, static_cast<int>(bytes));
+}
+
 constexpr size_t align_up(size_t x, size_t a) { return (x + a - 1) / a * a; }
 
 } // namespace psi

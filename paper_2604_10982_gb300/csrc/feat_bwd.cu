@@ -376,8 +376,9 @@ cudaError_t launch_reg(const FrameParams &fp, const FeatBwdArgs &a, cudaStream_t
 {
     const auto kernel = feat_bwd_reg_kernel<DT, KMAX>;
     const size_t dyn = static_cast<size_t>(pixel_warps(fp.tile_h)) * fp.top_k * 32 * kSetBytes;
-    if (dyn > 48 * 1024) {
-        const cudaError_t e = cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, static_cast<int>(dyn));
+    constexpr size_t most = static_cast<size_t>(kPixelWarps) * KMAX * 32 * kSetBytes;
+    if (most > 48 * 1024) {
+        const cudaError_t e = allow_dynamic_smem(kernel, most);
         if (e != cudaSuccess) return e;
     }
     kernel<<<static_cast<unsigned>(fp.n_tiles_total), 16 * fp.tile_h, dyn, st>>>(fp, a);

@@ -971,7 +971,7 @@ cudaError_t launch_kcslo(const FrameParams &fp, const FeatView &f, const BwdArgs
         if (f.data && f.dim == 16) {
             auto launch = [&](auto kernel) {
                 constexpr size_t dyn = feat_stage_bytes(16);
-                const cudaError_t e = cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, static_cast<int>(dyn));
+                const cudaError_t e = allow_dynamic_smem(kernel, dyn);
                 if (e != cudaSuccess) return e;
                 kernel<<<grid, nt, dyn, st>>>(fp, a);
                 return cudaGetLastError();

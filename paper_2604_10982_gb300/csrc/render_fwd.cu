@@ -471,13 +471,11 @@ cudaError_t launch_one(const FrameParams &fp, const FwdArgs &a, cudaStream_t st)
 {
     const auto kernel = render_fwd_kernel<KMAX, DT, CH, LP, OCC, TH>;
     const unsigned grid = a.work ? persistent_grid(fp.n_tiles_total, OCC) : fp.n_tiles_total;
-    const size_t dyn = KMAX > 0 ? static_cast<size_t>(pixel_warps(TH)) * topk_entries(fp.top_k) * sizeof(float4)
-                                : (a.feat ? feat_stage_bytes(CH) : 0);
-    if (dyn > 0) {
-        // the sets or features and the record stages together pass 48 KB
-        const cudaError_t e = cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, static_cast<int>(dyn));
-        if (e != cudaSuccess) return e;
-    }
+    auto set_bytes = [](int K) { return static_cast<size_t>(pixel_warps(TH)) * topk_entries(K) * sizeof(float4); };
+    const size_t dyn = KMAX > 0 ? set_bytes(fp.top_k) : (a.feat ? feat_stage_bytes(CH) : 0);
+    // the sets or features and the record stages together pass 48 KB
+    const cudaError_t e = allow_dynamic_smem(kernel, KMAX > 0 ? set_bytes(KMAX) : feat_stage_bytes(CH));
+    if (e != cudaSuccess) return e;
     kernel<<<grid, pipe_threads(TH), dyn, st>>>(fp, a);
     return cudaGetLastError();
 }

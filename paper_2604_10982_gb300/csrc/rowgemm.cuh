@@ -192,15 +192,17 @@ cudaError_t launch_row_gemm(const void *A, int64_t rows, int D, const void *B, i
     RowGemm p{rows, D, n_pad, status};
     // shared memory of at least 120 KB (one CTA per SM) or 80 KB (two): never
     // more CTAs on an SM than their 256 TMEM columns each can be granted at once
-    const size_t smem = std::max<size_t>(ctas == 1 ? 120 * 1024 : 80 * 1024,
-                                         1024 + static_cast<size_t>(kRowStages) * (D / 64) * kRowM * 128 +
-                                             static_cast<size_t>(D / 64) * n_pad * 128 + epi_smem_bytes);
+    auto smem_bytes = [&](int dim, int cols) {
+        return std::max<size_t>(ctas == 1 ? 120 * 1024 : 80 * 1024,
+                                1024 + static_cast<size_t>(kRowStages) * (dim / 64) * kRowM * 128 +
+                                    static_cast<size_t>(dim / 64) * cols * 128 + epi_smem_bytes);
+    };
+    const size_t smem = smem_bytes(D, n_pad);
     if (ctas == 2 && 3 * smem <= 228 * 1024) {
         *why = "row GEMM shared memory too small to keep a third CTA off the SM";
         return cudaErrorInvalidValue;
     }
-    cudaError_t e = cudaFuncSetAttribute(row_gemm_kernel<Epi>, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                                         static_cast<int>(smem));
+    cudaError_t e = allow_dynamic_smem(row_gemm_kernel<Epi>, smem_bytes(128, 128)); // epi_smem_bytes: one value per Epi
     if (e != cudaSuccess) return e;
     int dev = 0, sms = 0;
     cudaGetDevice(&dev);

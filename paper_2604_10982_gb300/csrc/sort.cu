@@ -501,8 +501,7 @@ cudaError_t launch_sort(uint64_t *keys, uint32_t *vals, const int64_t *d_num_pai
             plan.shift[ps] = begin_bit + ps * dbits;
             plan.bits[ps] = std::min(dbits, end_bit - plan.shift[ps]);
         }
-        const cudaError_t e = cudaFuncSetAttribute(small_sort_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                                                   static_cast<int>(sizeof(SmallSmem)));
+        const cudaError_t e = allow_dynamic_smem(small_sort_kernel, sizeof(SmallSmem));
         if (e != cudaSuccess) return e;
         small_sort_kernel<<<1, kSmallThreads, sizeof(SmallSmem), st>>>(keys, vals, d_num_pairs, cap, plan,
                                                                        want_ranges ? tile_ranges : nullptr,
@@ -534,8 +533,7 @@ cudaError_t launch_sort(uint64_t *keys, uint32_t *vals, const int64_t *d_num_pai
         plan.shift[ps] = bits == 0 ? 0 : shift; // identity pass (keeps the pass count even)
         plan.bits[ps] = bits;
     }
-    e = cudaFuncSetAttribute(onesweep_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                             static_cast<int>(sizeof(ScatterSmem)));
+    e = allow_dynamic_smem(onesweep_kernel, sizeof(ScatterSmem));
     if (e != cudaSuccess) return e;
     int dev = 0, sms = 148;
     cudaGetDevice(&dev);
