@@ -193,8 +193,7 @@ struct TopK {
 // waiting at a CTA barrier; released[w] counts the batches pixel warp w is
 // done with, so that a warp whose pixels are all saturated can leave the walk
 // (kLeft) and finish its pixels while the others composite, instead of
-// following the stream to its end. `alive` counts the warps still in the walk
-// (the producer stops at zero). Every wait is bounded; a waiting warp is
+// following the stream to its end (the producer stops when all have). Every wait is bounded; a waiting warp is
 // suspended in hardware.
 constexpr int kPB = 128;          // records per stage (four 32-bit hit words per warp)
 // pixel warps of a 16 x TH tile (8x4-pixel blocks, two per block row) and the
@@ -217,7 +216,6 @@ struct PipeT {
     uint32_t val[kPS][kPB];
     uint64_t ready[kPS]; // one arrival per pixel warp (the producer arrives for all of them)
     int released[kPixelWarps]; // batches each pixel warp is done with (unused ones: kLeft)
-    int alive;
     int abort;
     unsigned long long limit; // the context's wait limit (ns)
 };
@@ -226,17 +224,16 @@ using Pipe = PipeT<4>;
 
 __device__ __forceinline__ int vload(const int &x) { return *reinterpret_cast<const volatile int *>(&x); }
 
-// thread 0; the caller synchronises the CTA afterwards. alive = the number of
+// thread 0; the caller synchronises the CTA afterwards. warps = the number of
 // pixel warps (each releases every stage once per batch), limit = wait_limit()
 template <class PP>
-__device__ __forceinline__ void pipe_init(PP &P, int alive, unsigned long long limit)
+__device__ __forceinline__ void pipe_init(PP &P, int warps, unsigned long long limit)
 {
     P.limit = limit;
     for (int s = 0; s < PP::kPS; ++s) {
-        mbar_init(&P.ready[s], alive);
+        mbar_init(&P.ready[s], warps);
     }
-    for (int w = 0; w < kPixelWarps; ++w) P.released[w] = w < alive ? 0 : kLeft;
-    P.alive = alive;
+    for (int w = 0; w < kPixelWarps; ++w) P.released[w] = w < warps ? 0 : kLeft;
     P.abort = 0;
     fence_mbar_init();
 }
@@ -408,11 +405,50 @@ __device__ __forceinline__ void pipe_prefill(PP &P, int w, const uint32_t *__res
     if (lane == 0) mbar_arrive_n(&P.ready[b], kShare);
 }
 
+// Batches that every pixel warp in the walk is done with: kLeft when all have
+// left it, -1 after an abort. One answer for the whole (producer) warp, as the
+// warp-wide operations of its loop need; lane w has acquired warp w's release.
+template <class PP>
+__device__ __forceinline__ int pipe_progress(const PP &P)
+{
+    const int lane = threadIdx.x & 31;
+    int done = kLeft;
+    if (lane < kPixelWarps)
+        done = ld_acquire_cta_shared(&P.released[lane]);
+    else if (lane == kPixelWarps && vload(P.abort))
+        done = -1;
+    return __reduce_min_sync(0xffffffffu, done);
+}
+
+// Producer warp: waits until the stage of batch b is free (every pixel warp is
+// done with the batch before it there). False if there is nothing more to
+// stage for: every warp has left, or an abort -- its own, when the wait runs
+// out. One exit, for all lanes together.
+template <class PP>
+__device__ __forceinline__ bool pipe_wait_free(PP &P, int b, DevStatus *st, int site)
+{
+    unsigned long long t0 = 0;
+    int done = pipe_progress(P);
+    while (done >= 0 && done <= b - PP::kPS) {
+        if (wait_expired(t0, P.limit)) {
+            if (st) {
+                atomicCAS(&st->wait_site, 0, site);
+                raise_status(st, PSI_ERR_TIMEOUT);
+            }
+            atomicExch(&P.abort, 1);
+        }
+        __nanosleep(64);
+        done = pipe_progress(P);
+    }
+    __syncwarp(); // what one lane acquired orders every lane's refill of the stage
+    return done >= 0 && done != kLeft;
+}
+
 // Producer warp: stages the batches after the prefilled ones of the list
-// (entries [list0, list0+n)), forward or reverse, until all are staged or no
-// pixel warp is alive. Returns false on a timeout (status raised, abort set).
+// (entries [list0, list0+n)), forward or reverse, until all are staged, every
+// pixel warp has left the walk, or a wait runs out (status raised, abort set).
 template <bool LP, int PW, class PP, class Extra = NoExtra>
-__device__ __forceinline__ bool pipe_produce(PP &P, const uint32_t *__restrict__ vals, int64_t list0, int n,
+__device__ __forceinline__ void pipe_produce(PP &P, const uint32_t *__restrict__ vals, int64_t list0, int n,
                                              bool reverse, const float4 *__restrict__ records, int tile_x0,
                                              int tile_y0, DevStatus *st, int site, uint32_t rec_lo, uint32_t rec_hi,
                                              const Extra &extra = Extra())
@@ -431,33 +467,12 @@ __device__ __forceinline__ bool pipe_produce(PP &P, const uint32_t *__restrict__
         return true;
     };
     int c = prefill_batches<PW>() * kChunks;
-    if (c >= nb * kChunks) return true;
     uint32_t i0 = 0, i1 = 0; // this chunk's and the next chunk's record index
     bool v0 = entry(c, i0), v1 = entry(c + 1, i1);
 #pragma unroll 1
     for (; c < nb * kChunks; ++c) {
         const int b = c / kChunks, s = b % PP::kPS;
-        if (c % kChunks == 0 && b >= PP::kPS) {
-            // the stage's last batch must have been released by every pixel warp
-            unsigned long long t0 = 0;
-            while (true) {
-                if (vload(P.alive) == 0 || vload(P.abort)) return true;
-                const int done = lane < kPixelWarps ? ld_acquire_cta_shared(&P.released[lane]) : kLeft;
-                if (__reduce_min_sync(0xffffffffu, done) > b - PP::kPS) break;
-                const unsigned long long now = global_ns();
-                if (t0 == 0) {
-                    t0 = now;
-                } else if (now - t0 > P.limit) {
-                    if (lane == 0 && st) {
-                        atomicCAS(&st->wait_site, 0, site);
-                        raise_status(st, PSI_ERR_TIMEOUT);
-                    }
-                    if (lane == 0) atomicExch(&P.abort, 1);
-                    return false;
-                }
-                __nanosleep(64);
-            }
-        }
+        if (c % kChunks == 0 && !pipe_wait_free(P, b, st, site)) return;
         const int j = (c % kChunks) * 32 + lane;
         if (v1) prefetch_record(records, i1);
         if (v0) {
@@ -471,10 +486,8 @@ __device__ __forceinline__ bool pipe_produce(PP &P, const uint32_t *__restrict__
         if (c % kChunks == kChunks - 1) {
             __syncwarp();
             if (lane == 0) mbar_arrive_n(&P.ready[s], PW);
-            if (vload(P.alive) == 0 || vload(P.abort)) return true;
         }
     }
-    return true;
 }
 
 // Pixel warp (all 32 lanes): wait until batch b is ready. Returns false
@@ -525,10 +538,7 @@ template <class PP>
 __device__ __forceinline__ void pipe_leave(PP &P, int w)
 {
     __syncwarp();
-    if ((threadIdx.x & 31) == 0) {
-        st_release_cta_shared(&P.released[w], kLeft);
-        atomicSub(&P.alive, 1);
-    }
+    if ((threadIdx.x & 31) == 0) st_release_cta_shared(&P.released[w], kLeft);
 }
 
 // The records of one staged batch that can reach a pixel of each group of

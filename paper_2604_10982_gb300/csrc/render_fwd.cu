@@ -365,7 +365,9 @@ __device__ __forceinline__ void fwd_tile(const FrameParams &fp, const FwdArgs &a
             pipe_release(P, wid, b);
         }
     }
-    if (vload(P.abort)) return;
+    // one answer for the warp, whose gather is warp-wide (as a vote, which the
+    // compiler knows to be uniform, 1.3 % slower at K = 8)
+    if (__shfl_sync(0xffffffffu, vload(P.abort), 0)) return;
 
     const int64_t pix = cam.pix_base + static_cast<int64_t>(py) * cam.W + px;
     if (inside && a.write_rgb) {
