@@ -40,7 +40,6 @@ __device__ __forceinline__ float rcp_approx(float x)
 // ((w & 1) * 8, (w >> 1) * 4). Its four groups of eight consecutive lanes
 // own the block's 4x2 quarters: group g = l >> 3 is the quarter at
 // ((g >> 1) * 4, (g & 1) * 2), lane l pixel (l & 3, (l >> 2) & 1) of it.
-constexpr int kGroups = 4;
 __device__ __forceinline__ void pixel_of_thread(int tid, int &lx, int &ly)
 {
     const int w = tid >> 5, l = tid & 31;
@@ -206,7 +205,7 @@ constexpr int kPipeThreads = pipe_threads(16);
 constexpr int kLeft = 0x7fffffff;  // released[w] of a warp that left the walk
 constexpr uint32_t kSuspendNs = 20000; // longest hardware suspension per poll of a wait
 
-// NS stages: 4, or 3 where a fourth costs a resident CTA (with two of them
+// NS stages: 4, or 3 where a fourth costs a resident CTA or the L1 (with two of them
 // prefilled, each further one lets a fast warp run ahead of a slow one: 4
 // against 3 is 0.90 against 1.00 ms for the adjoint of the depth/normal maps)
 template <int NS>
@@ -221,6 +220,20 @@ struct PipeT {
 };
 
 using Pipe = PipeT<4>;
+
+// Index lists of a warp's groups (build_hits), and whether `occ` CTAs of a
+// compositing kernel -- stages, lists, `dyn` bytes of dynamic shared memory,
+// 16 bytes of its own and the 1 KB the system takes -- fit an SM's shared memory. The
+// launches assert it for the CTAs per SM that their build is for: one CTA fewer
+// than that runs with the registers of more, and a persistent grid would hold
+// CTAs that start only when the others have finished.
+constexpr int kGroups = 4;
+using HitLists = uint8_t[kGroups][kPB];
+template <class PP>
+constexpr bool smem_fits(int occ, int TH, size_t dyn)
+{
+    return occ * (sizeof(PP) + sizeof(HitLists) * pixel_warps(TH) + 16 + dyn + 1024) <= 228 * 1024;
+}
 
 __device__ __forceinline__ int vload(const int &x) { return *reinterpret_cast<const volatile int *>(&x); }
 
@@ -548,8 +561,7 @@ __device__ __forceinline__ void pipe_leave(PP &P, int w)
 // records that meet its 8x4 block. On a 1080p street of 3M surfels (median
 // splat 8 pixels wide) that is 8.3M against 16.4M trips before the first
 // pixel saturates.
-using HitLists = uint8_t[kGroups][kPB];
-
+//
 // Builds the lists of pixel warp vw (its block's place in the 16x16 tile) for
 // the first `cnt` records of stage s, taking record j into group g's list
 // only if j < lim[g]; n[g] = length. NG = 4: one list per group; NG = 1: one

@@ -231,8 +231,8 @@ __device__ __forceinline__ void group_transpose_sum16(float v[16], int lane)
 // rounds, which would leave 28 of 32 lanes idle at 16 channels.
 // Pass B walks one list per group of lanes (build_hits) unless the feature
 // gradient is summed by the whole warp, lanes across channels (NG = 1).
-template <int KMAX, int DT, int CH, bool SAVED, bool LP, int TH, bool NW = false>
-__device__ __forceinline__ void bwd_tile(const FrameParams &fp, const BwdArgs &a, Pipe &P, HitLists *hits,
+template <int KMAX, int DT, int CH, bool SAVED, bool LP, int TH, bool NW = false, class PP>
+__device__ __forceinline__ void bwd_tile(const FrameParams &fp, const BwdArgs &a, PP &P, HitLists *hits,
                                          int &s_maxlast, float4 *feat_stage, uint32_t tile)
 {
     constexpr int PW = pixel_warps(TH);
@@ -297,7 +297,7 @@ __device__ __forceinline__ void bwd_tile(const FrameParams &fp, const BwdArgs &a
         if (!in_walk) pipe_leave(P, wid);
         for (int b = 0; b < nb && in_walk; ++b) {
             if (!pipe_wait_ready(P, b, a.status, kSiteRenderBwdA)) break;
-            const int st = b % Pipe::kPS;
+            const int st = b % PP::kPS;
             int cnt;
             const int lo = batch_range(b, n, false, cnt);
             int ng[kGroups];
@@ -383,7 +383,7 @@ __device__ __forceinline__ void bwd_tile(const FrameParams &fp, const BwdArgs &a
         if (vload(P.abort)) return;
         if (tid == 0) {
             // fresh barriers for the reverse walk
-            for (int s = 0; s < Pipe::kPS; ++s) {
+            for (int s = 0; s < PP::kPS; ++s) {
                 asm volatile("mbarrier.inval.shared::cta.b64 [%0];" ::"r"(smem_u32(&P.ready[s])) : "memory");
             }
             pipe_init(P, PW, P.limit);
@@ -429,7 +429,7 @@ __device__ __forceinline__ void bwd_tile(const FrameParams &fp, const BwdArgs &a
     const bool want_feat = !ext_feat && a.g_F && a.g_feat;
     for (int b = 0; b < nbB; ++b) {
         if (!pipe_wait_ready(P, b, a.status, kSiteRenderBwdB)) break;
-        const int st = b % Pipe::kPS;
+        const int st = b % PP::kPS;
         int cnt;
         const int lo = batch_range(b, maxlast, true, cnt);
         int ng[NG], lim[NG];
@@ -812,6 +812,11 @@ __global__ void __launch_bounds__(pair_threads(TH), OCC)
     }
 }
 
+// Record stages: with four, five CTAs of a 16x8 tile take nearly all of the SM's
+// shared memory and with it the L1 (3M-surfel 1080p frame, K = 8, saved state:
+// adjoint 3.38 against 2.78 ms).
+__host__ __device__ constexpr int bwd_stages(int TH) { return TH == 8 ? 3 : 4; }
+
 // OCC: CTAs per SM the kernel is built for (the launch shape the autotuner
 // picks). Tiles longest list first; the persistent launch (a.work set) fetches
 // further tiles from the context's counter as the forward kernel does.
@@ -819,7 +824,7 @@ template <int KMAX, int DT, int CH, bool SAVED, bool LP, int OCC, int TH = 16, b
 __global__ void __launch_bounds__(pipe_threads(TH), OCC)
     render_bwd_kernel(const __grid_constant__ FrameParams fp, BwdArgs a)
 {
-    __shared__ __align__(128) Pipe P;
+    __shared__ __align__(128) PipeT<bwd_stages(TH)> P;
     __shared__ HitLists hits[pixel_warps(TH)];
     extern __shared__ __align__(16) float4 feat_stage[]; // NW: feat_stage_bytes(16)
     __shared__ int s_maxlast;
@@ -966,6 +971,8 @@ cudaError_t launch_kcslo(const FrameParams &fp, const FeatView &f, const BwdArgs
     unsigned grid = fp.n_tiles_total;
     if (a.work) grid = persistent_grid(fp.n_tiles_total, OCC);
     constexpr int nt = pipe_threads(TH);
+    static_assert(smem_fits<PipeT<bwd_stages(TH)>>(OCC, TH, KMAX == 0 && CH == 16 ? feat_stage_bytes(16) : 0),
+                  "fewer CTAs fit than the build is for");
     if constexpr (KMAX == 0 && CH == 16) {
         // dense 16-channel tables: the register-held g_F row, the table's rows staged with the records
         if (f.data && f.dim == 16) {
@@ -993,9 +1000,10 @@ cudaError_t launch_kcslo(const FrameParams &fp, const FeatView &f, const BwdArgs
     return cudaGetLastError();
 }
 
-// 16x8 tiles (Top-K with K <= 8, no low-pass filter): 4 pixel warps, 5 CTAs per SM
-// (shared memory: one pipeline each)
-constexpr int kOccTile8 = 5;
+// 16x8 tiles (Top-K with K <= 8, no low-pass filter): 4 pixel warps, 5 CTAs per SM,
+// 4 when pass A recomputes the set (the 5-CTA build spills and reads feature rows
+// through what is left of the L1: 6.62 against 5.67 ms, K = 8, 3M-surfel 1080p frame)
+constexpr int kOccTile8 = 5, kOccTile8Recompute = 4;
 
 template <int KMAX, int CH, bool SAVED, bool LP>
 cudaError_t launch_kcsl(const FrameParams &fp, const FeatView &f, const BwdArgs &a, bool alt, cudaStream_t st)
@@ -1117,7 +1125,7 @@ cudaError_t launch_render_bwd(const FrameParams &fp, const psi_surfels &s, const
         e = launch_pair(fp, a, alt, st);
     else if (fp.tile_h == 8)
         e = a.saved_T ? launch_kcslo<8, 16, true, false, kOccTile8, 8>(fp, f, a, st)
-                      : launch_kcslo<8, 16, false, false, kOccTile8, 8>(fp, f, a, st);
+                      : launch_kcslo<8, 16, false, false, kOccTile8Recompute, 8>(fp, f, a, st);
     else if (K == 0)
         e = ch == 32 ? launch_dense<32>(fp, f, a, alt, st) : launch_dense<16>(fp, f, a, alt, st);
     else if (a.saved_T)

@@ -126,7 +126,7 @@ struct TopKShared {
 };
 
 // float4 of shared memory per warp for the sets: K rounded up to four slots
-__host__ __device__ inline int topk_entries(int K) { return (K + 3) / 4 * 64; }
+__host__ __device__ constexpr int topk_entries(int K) { return (K + 3) / 4 * 64; }
 
 // The Top-K feature sum of the warp's 32 pixels, F = scale * sum_{j in K}
 // omega_j q_j, and / or its channel argmax. ent holds each pixel's selection
@@ -430,6 +430,16 @@ __device__ __forceinline__ void fwd_tile(const FrameParams &fp, const FwdArgs &a
     }
 }
 
+// Record stages: four where the CTAs per SM that the build is for fit with them
+// (K <= 8 at three, dense features). With the sets (2 KB per slot and 16x16 tile,
+// half for 16x8) four stages let only three of four and four of five CTAs be
+// resident: 1.58 against 1.51 ms at four CTAs, 1.63 against 1.44 ms for 16x8
+// tiles at five (3M-surfel 1080p frame, K = 8; three CTAs and four stages: 1.46).
+__host__ __device__ constexpr int fwd_stages(int KMAX, int OCC, int TH)
+{
+    return KMAX > 8 || (KMAX > 0 && (OCC > 3 || TH == 8)) ? 3 : 4;
+}
+
 // OCC: CTAs per SM the kernel is built for (the launch shape the autotuner
 // picks). Tiles are taken longest list first: CTA b starts with entry b of the
 // launch order; in the persistent launch (a.work set, grid of a few CTAs per
@@ -440,7 +450,7 @@ template <int KMAX, int DT, int CH, bool LP, int OCC, int TH = 16>
 __global__ void __launch_bounds__(pipe_threads(TH), OCC)
     render_fwd_kernel(const __grid_constant__ FrameParams fp, FwdArgs a)
 {
-    __shared__ __align__(128) PipeT<(KMAX > 8 ? 3 : 4)> P;
+    __shared__ __align__(128) PipeT<fwd_stages(KMAX, OCC, TH)> P;
     __shared__ HitLists hits[pixel_warps(TH)];
     __shared__ uint32_t s_next;
     extern __shared__ __align__(16) float4 entries[]; // K > 0: topk_entries(K) per pixel warp; dense: feature stages
@@ -473,10 +483,12 @@ cudaError_t launch_one(const FrameParams &fp, const FwdArgs &a, cudaStream_t st)
 {
     const auto kernel = render_fwd_kernel<KMAX, DT, CH, LP, OCC, TH>;
     const unsigned grid = a.work ? persistent_grid(fp.n_tiles_total, OCC) : fp.n_tiles_total;
-    auto set_bytes = [](int K) { return static_cast<size_t>(pixel_warps(TH)) * topk_entries(K) * sizeof(float4); };
+    constexpr auto set_bytes = [](int K) constexpr { return static_cast<size_t>(pixel_warps(TH)) * topk_entries(K) * sizeof(float4); };
     const size_t dyn = KMAX > 0 ? set_bytes(fp.top_k) : (a.feat ? feat_stage_bytes(CH) : 0);
+    constexpr size_t most = KMAX > 0 ? set_bytes(KMAX) : feat_stage_bytes(CH);
+    static_assert(smem_fits<PipeT<fwd_stages(KMAX, OCC, TH)>>(OCC, TH, most), "fewer CTAs fit than the build is for");
     // the sets or features and the record stages together pass 48 KB
-    const cudaError_t e = allow_dynamic_smem(kernel, KMAX > 0 ? set_bytes(KMAX) : feat_stage_bytes(CH));
+    const cudaError_t e = allow_dynamic_smem(kernel, most);
     if (e != cudaSuccess) return e;
     kernel<<<grid, pipe_threads(TH), dyn, st>>>(fp, a);
     return cudaGetLastError();
@@ -492,7 +504,7 @@ cudaError_t launch_kclo(const FrameParams &fp, const FeatView &f, const FwdArgs 
     }
 }
 
-// 16x8 tiles (Top-K with K <= 8, no low-pass filter): 4 pixel warps, up to 5 CTAs per SM
+// 16x8 tiles (Top-K with K <= 8, no low-pass filter): 4 pixel warps, 5 CTAs per SM
 constexpr int kOccTile8 = 5;
 
 template <int KMAX, int CH, bool LP>

@@ -74,3 +74,49 @@ def test_warps_leave_the_walk_at_different_batches(ctx, K, lowpass):
         for which, saved in ((0, 0), (1, 1), (1, 0)):
             psi.psi_ctx_set_render_shape(ctx, which, r.opts, psi.F32, saved, 0)
     assert ctx.status_fetch() == (0, 0)
+
+
+FORMS = {  # options, feature dim, forward shape, adjoint shapes from saved state, recomputing
+    "tile8": (dict(top_k=8, tile_h=8), 32, 0, (0, 4), (0, 4)),
+    "tile8_k3": (dict(top_k=3, tile_h=8), 32, 4, (0,), (0,)),
+    "tile8_pair": (dict(top_k=8, tile_h=8), 32, 0, (8, 12), (0,)),
+    "alternative": (dict(top_k=8), 32, 1, (1,), (1,)),
+    "alternative_persistent": (dict(top_k=8), 32, 5, (5, 13), (5,)),
+    "lowpass": (dict(top_k=8, lowpass=True), 32, 1, (0, 1, 8), (0,)),
+    "dense32": (dict(top_k=0), 32, 0, (0, 1), (0,)),
+}
+
+
+@pytest.mark.parametrize("n", [127, 129, 257, 513, 900])
+@pytest.mark.parametrize("form", list(FORMS))
+def test_forms_at_list_lengths(ctx, form, n):
+    """Forward against the oracle (this input excuses no pixel), bit for bit
+    against the default shape; every adjoint form against the default one."""
+    from paper_2604_10982_gb300 import pipeline as pl, psi
+    kw, D, fwd, saved_shapes, re_shapes = FORMS[form]
+    w = _stack(n, D)
+    cam = w.cameras[0]
+    o = orc.Opts(mode=orc.EXACT, opacity_radius=True, **kw)
+    scene = pl.DeviceScene(w.surfels, w.features)
+    base = pl.make_renderer(ctx, scene, [cam], opts_of(orc.Opts(mode=orc.EXACT, opacity_radius=True,
+                                                                **{k: v for k, v in kw.items() if k != "tile_h"})), D=D)
+    base.frame(scene)
+    up = _upstream(base.n_pix, D)
+    g0 = base.backward(scene, *up)
+    r = pl.make_renderer(ctx, scene, [cam], opts_of(o), D=D)
+    try:
+        psi.psi_ctx_set_render_shape(ctx, 0, r.opts, psi.F32, 0, fwd)
+        r.frame(scene)
+        ref = orc.render(w.surfels, cam, o, feat=w.features.astype(np.float64))
+        check_values(r.rgb.cpu().numpy().astype(np.float64).T, r.T.cpu().numpy().astype(np.float64),
+                     r.F.cpu().numpy().astype(np.float64), ref, cam, max_excused=0, fmax=np.abs(w.features).max())
+        for name in ("rgb", "T", "F") + (("topk_ids", "topk_w") if kw["top_k"] else ()):
+            assert torch.equal(getattr(r, name), getattr(base, name)), name
+        for saved, shapes in ((1, saved_shapes), (0, re_shapes)):
+            for shape in shapes:
+                psi.psi_ctx_set_render_shape(ctx, 1, r.opts, psi.F32, saved, shape)
+                _close(r.backward(scene, *up, recompute=not saved), g0, (saved, shape))
+    finally:
+        for which, saved in ((0, 0), (1, 1), (1, 0)):
+            psi.psi_ctx_set_render_shape(ctx, which, r.opts, psi.F32, saved, 0)
+    assert ctx.status_fetch() == (0, 0)
