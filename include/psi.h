@@ -276,6 +276,9 @@ int psi_sort_keys(psi_ctx *ctx, uint64_t *keys, uint32_t *vals, const int64_t *d
                   int begin_bit, int end_bit, uint32_t *tile_ranges, int64_t n_tiles_total, void *workspace,
                   size_t workspace_bytes, psi_stream stream);
 
+/* Kernels that psi_sort_keys launches for these sizes (memsets excluded). */
+int psi_sort_kernel_count(int64_t capacity, int begin_bit, int end_bit, int64_t n_tiles_total, int *kernels);
+
 /* ---- a3 without caller scratch (no counterpart in the paper) ------------
  * Same result as psi_sort_keys, for callers that cannot allocate device memory
  * for a workspace: real-time loops that must not stall on an allocator, or

@@ -265,6 +265,14 @@ int psi_sort_workspace_size(int64_t capacity, size_t *bytes)
     return PSI_OK;
 }
 
+int psi_sort_kernel_count(int64_t capacity, int begin_bit, int end_bit, int64_t n_tiles_total, int *kernels)
+{
+    if (!kernels || capacity < 0 || begin_bit < 0 || end_bit > 64 || begin_bit >= end_bit || n_tiles_total < 0)
+        return PSI_ERR_INVALID_ARG;
+    *kernels = psi::sort_kernel_count(capacity, begin_bit, end_bit, n_tiles_total);
+    return PSI_OK;
+}
+
 int psi_render_bwd_workspace_size(int64_t n_records, int64_t n_pix, int top_k, size_t *bytes)
 {
     if (!bytes || n_records < 0 || n_pix < 0 || top_k < 0 || top_k > PSI_MAX_TOPK) return PSI_ERR_INVALID_ARG;

@@ -259,6 +259,7 @@ cudaError_t launch_intersect(const FrameParams &fp, const float4 *bin_records, c
                              DevStatus *status, cudaStream_t st);
 
 size_t sort_workspace_bytes(int64_t capacity);
+int sort_kernel_count(int64_t capacity, int begin_bit, int end_bit, int64_t n_tiles_total);
 cudaError_t launch_sort(uint64_t *keys, uint32_t *vals, const int64_t *d_num_pairs, int64_t capacity, int begin_bit,
                         int end_bit, uint32_t *tile_ranges, int64_t n_tiles_total, void *ws, DevStatus *status,
                         cudaStream_t st);

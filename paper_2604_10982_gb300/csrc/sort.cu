@@ -474,6 +474,20 @@ __global__ void __launch_bounds__(kSmallThreads) small_sort_kernel(uint64_t *key
 } // namespace
 
 namespace {
+// whether launch_sort takes the one-CTA kernel
+bool one_cta(int64_t cap, bool want_ranges, int64_t n_tiles)
+{
+    return cap <= kSmallPairs && (!want_ranges || n_tiles <= kSmallTiles);
+}
+
+// the general path: an even number of passes, so that the result ends in the
+// caller's buffers
+int general_passes(int nbits)
+{
+    const int passes = std::max(2, (nbits + 7) / 8);
+    return passes + (passes & 1);
+}
+
 int64_t sort_partitions(int64_t capacity) { return (std::max<int64_t>(capacity, 1) + kTile - 1) / kTile; }
 } // namespace
 
@@ -486,6 +500,14 @@ size_t sort_workspace_bytes(int64_t capacity)
            align_up(sort_partitions(cap) * kBins * 8, 256);
 }
 
+int sort_kernel_count(int64_t capacity, int begin_bit, int end_bit, int64_t n_tiles_total)
+{
+    const bool want_ranges = n_tiles_total > 0;
+    if (one_cta(std::max<int64_t>(capacity, 1), want_ranges, n_tiles_total)) return 1;
+    // digit counts, digit scan, the passes; ranges and tile order
+    return 2 + general_passes(std::max(end_bit - begin_bit, 1)) + (want_ranges ? 2 : 0);
+}
+
 cudaError_t launch_sort(uint64_t *keys, uint32_t *vals, const int64_t *d_num_pairs, int64_t capacity, int begin_bit,
                         int end_bit, uint32_t *tile_ranges, int64_t n_tiles_total, void *ws, DevStatus *status,
                         cudaStream_t st)
@@ -493,7 +515,7 @@ cudaError_t launch_sort(uint64_t *keys, uint32_t *vals, const int64_t *d_num_pai
     const int64_t cap = std::max<int64_t>(capacity, 1);
     const int nbits = std::max(end_bit - begin_bit, 1);
     const bool want_ranges = tile_ranges && n_tiles_total > 0;
-    if (cap <= kSmallPairs && (!want_ranges || n_tiles_total <= kSmallTiles)) {
+    if (one_cta(cap, want_ranges, n_tiles_total)) {
         PassPlan plan{};
         plan.passes = (nbits + 7) / 8;
         const int dbits = (nbits + plan.passes - 1) / plan.passes;
@@ -524,8 +546,7 @@ cudaError_t launch_sort(uint64_t *keys, uint32_t *vals, const int64_t *d_num_pai
     if (e != cudaSuccess) return e;
 
     PassPlan plan{};
-    plan.passes = std::max(2, (nbits + 7) / 8);
-    if (plan.passes & 1) ++plan.passes;
+    plan.passes = general_passes(nbits);
     const int dbits = (nbits + plan.passes - 1) / plan.passes;
     for (int ps = 0; ps < plan.passes; ++ps) {
         const int shift = begin_bit + ps * dbits;

@@ -137,13 +137,7 @@ class Renderer:
         R = self.V * self.n
         n = 1 if R else 0                                  # project
         n += 1 if R else 0                                 # intersect
-        if self.capacity <= 8192 and self.n_tiles <= 16384:
-            n += 1                                         # the one-CTA sort with ranges and tile order
-        else:
-            nbits = max(self.key_bits, 1)
-            passes = max(2, (nbits + 7) // 8)
-            passes += passes & 1
-            n += passes + 4                                # digit counts, digit scan, one pass each, ranges, tile order
+        n += psi.sort_kernel_count(self.capacity, 0, self.key_bits, self.n_tiles)
         K = int(self.opts.top_k)
         D = self.D
         ch = 32 if D % 32 == 0 else 16

@@ -86,6 +86,7 @@ def lib():
         L.psi_view_layout.argtypes = [ctypes.POINTER(PsiCamera), ctypes.c_int, ctypes.POINTER(PsiRenderOpts), _P, _P]
         for f in ("psi_intersect_workspace_size", "psi_sort_workspace_size"):
             getattr(L, f).argtypes = [_i64, ctypes.POINTER(sz)]
+        L.psi_sort_kernel_count.argtypes = [_i64, ctypes.c_int, ctypes.c_int, _i64, ctypes.POINTER(ctypes.c_int)]
         L.psi_render_bwd_workspace_size.argtypes = [_i64, _i64, ctypes.c_int, ctypes.POINTER(sz)]
         L.psi_project_surfels.argtypes = [_P, ctypes.POINTER(PsiSurfels), ctypes.POINTER(PsiCamera), ctypes.c_int,
                                           ctypes.POINTER(PsiRenderOpts), _P, _P, _P, _P]
@@ -238,6 +239,14 @@ def intersect_workspace_size(n_records):
 
 def sort_workspace_size(capacity):
     return _ws("psi_sort_workspace_size", capacity)
+
+
+def sort_kernel_count(capacity, begin_bit, end_bit, n_tiles):
+    k = ctypes.c_int(0)
+    rc = lib().psi_sort_kernel_count(int(capacity), begin_bit, end_bit, int(n_tiles), ctypes.byref(k))
+    if rc:
+        raise PsiError(rc, "psi_sort_kernel_count")
+    return k.value
 
 
 def render_bwd_workspace_size(n_records, n_pix=0, top_k=0):
