@@ -334,7 +334,9 @@ int psi_render_fwd(psi_ctx *ctx, const psi_features *f, const void *records, con
  *  PSI_ERR_INVALID_ARG). With them the feature part of the adjoint (<gF, f_j>
  *  and dL/df) runs per pixel from the saved selection, outside the list walk.
  *  Outputs that do not belong to this frame give wrong gradients; nothing
- *  checks that.
+ *  checks that, but an id outside the table counts as an empty slot and
+ *  n_last is cut to the tile's list, so nothing is read out of range (as after
+ *  a forward that gave up, which leaves the outputs of its tiles unwritten).
  *  workspace: psi_render_bwd_workspace_size(n_views*N, P_total, top_k) bytes. */
 int psi_render_bwd(psi_ctx *ctx, const psi_surfels *s, const psi_features *f, const void *records,
                    const uint32_t *vals, const uint32_t *tile_ranges, const psi_camera *cams, int n_views,

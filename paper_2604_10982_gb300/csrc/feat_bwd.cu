@@ -94,7 +94,7 @@ struct SlotOrder<KMAX, true> {
 };
 
 // The pixel's saved set sorted by surfel id (odd-even transposition
-// network; empty slots hold 0xffffffff and sort last), with each slot's
+// network; empty slots and ids outside the table hold 0xffffffff and sort last), with each slot's
 // weight and its index in the saved set.
 template <int KMAX, class Order>
 __device__ __forceinline__ void load_sorted_set(const FrameParams &fp, const FeatBwdArgs &a, bool inside, int64_t pix,
@@ -105,8 +105,10 @@ __device__ __forceinline__ void load_sorted_set(const FrameParams &fp, const Fea
 #pragma unroll
     for (int s = 0; s < KMAX; ++s) {
         int i = (inside && s < K) ? a.topk_ids[pix * K + s] : -1;
-        // debug builds: a saved id must be -1 or a surfel of the table
-        if (!PSI_CHECK(i >= -1 && i < fp.n, kChkFeatRow, a.status)) i = -1;
+        // a saved id must be -1 or a surfel of the table (debug builds report it):
+        // a forward that gave up leaves the slots of its tiles as they were
+        const bool known = i >= -1 && i < fp.n;
+        if (!PSI_CHECK(known, kChkFeatRow, a.status) || !known) i = -1;
         id[s] = static_cast<uint32_t>(i);
         w[s] = i >= 0 ? a.topk_w[pix * K + s] : 0.0f;
         if (inside && s < K && i < 0) a.sel[pix * K + s] = make_uint2(0xffffffffu, 0u);
