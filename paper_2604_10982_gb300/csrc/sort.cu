@@ -347,19 +347,13 @@ __global__ void __launch_bounds__(1024) tile_order_kernel(const uint32_t *ranges
 // one kernel of one CTA, the pairs held in shared memory between the passes.
 // The general path is 10 kernels and two memsets whatever the count: with the
 // one-kernel intersect this takes a preview frame of about a thousand pairs
-// from 119 to 49 us. The lines, by the time of the sort alone with all pairs
-// in use (one CTA / general, in us): 1000 pairs, 300 tiles 24 / 82 launched one
-// by one and 22 / 60 in a graph; 8192 pairs, 300 tiles 70 / 87 and 67 / 69;
-// 8192 pairs, 4096 tiles 74 / 91 and 71 / 68. Beyond, the one SM would hold a
-// replayed frame up longer than ten small launches. It also walks the tiles alone
-// (1 us per 1024): 6144 pairs, 16384 tiles 74 / 101 and 72 / 77, but 8192 pairs, 16384
-// tiles 88 / 104 and 86 / 78.
+// from 119 to 49 us. Above 8192 pairs the one SM would hold the frame up
+// longer than the launches.
 constexpr int kSmallThreads = 1024;
 constexpr int kSmallWarps = kSmallThreads / 32;
 constexpr int kSmallItems = 8;
 constexpr int kSmallPairs = kSmallThreads * kSmallItems; // 8192
 constexpr int64_t kSmallTiles = 16384;                   // tiles ranged and ordered by the one CTA
-constexpr int64_t kManyTiles = 4096, kManyTilesPairs = 6144; // above this many tiles: up to this many pairs
 
 struct SmallSmem {
     uint64_t keys[kSmallPairs];
@@ -483,8 +477,7 @@ namespace {
 // whether launch_sort takes the one-CTA kernel
 bool one_cta(int64_t cap, bool want_ranges, int64_t n_tiles)
 {
-    if (!want_ranges || n_tiles <= kManyTiles) return cap <= kSmallPairs;
-    return cap <= kManyTilesPairs && n_tiles <= kSmallTiles;
+    return cap <= kSmallPairs && (!want_ranges || n_tiles <= kSmallTiles);
 }
 
 // the general path: an even number of passes, so that the result ends in the

@@ -120,29 +120,3 @@ def test_forms_at_list_lengths(ctx, form, n):
         for which, saved in ((0, 0), (1, 1), (1, 0)):
             psi.psi_ctx_set_render_shape(ctx, which, r.opts, psi.F32, saved, 0)
     assert ctx.status_fetch() == (0, 0)
-
-
-@pytest.mark.parametrize("capacity,n_tiles", [(6144, 4097), (6145, 4097), (6144, 16384), (6144, 16385), (8192, 4096), (8192, 4097)])
-def test_sort_forms_with_many_tiles(ctx, capacity, n_tiles):
-    """Both sort forms where the number of tiles decides between them."""
-    from paper_2604_10982_gb300 import psi
-    rng = np.random.default_rng(n_tiles)
-    tile = rng.integers(0, n_tiles, capacity).astype(np.uint64)
-    keys = (tile << np.uint64(32)) | rng.integers(0, 50, capacity).astype(np.uint64)
-    k = torch.from_numpy(keys.view(np.int64)).cuda()
-    v = torch.arange(capacity, dtype=torch.int32, device="cuda")
-    num = torch.tensor([capacity], dtype=torch.int64, device="cuda")
-    ranges = torch.full((3 * n_tiles,), -1, dtype=torch.int32, device="cuda")
-    ws = torch.empty(psi.sort_workspace_size(capacity), dtype=torch.uint8, device="cuda")
-    psi.psi_sort_keys(ctx, k, v, num, capacity, 0, 47, ranges, n_tiles, ws)
-    assert ctx.status_fetch() == (0, 0)
-    order = np.argsort(keys, kind="stable")
-    assert np.array_equal(k.cpu().numpy().view(np.uint64), keys[order])
-    assert np.array_equal(v.cpu().numpy(), order.astype(np.int32))
-    rg = ranges.cpu().numpy().view(np.uint32).astype(np.int64)
-    ends = np.cumsum(np.bincount(tile.astype(np.int64), minlength=n_tiles))
-    some = np.diff(ends, prepend=0) > 0
-    assert np.array_equal(rg[1:2 * n_tiles:2][some], ends[some])
-    assert np.array_equal(rg[:2 * n_tiles:2][some], np.concatenate([[0], ends[:-1]])[some])
-    assert (rg[:2 * n_tiles].reshape(-1, 2)[~some] == 0).all()
-    assert np.array_equal(np.sort(rg[2 * n_tiles:]), np.arange(n_tiles))
