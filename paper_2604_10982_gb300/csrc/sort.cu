@@ -347,8 +347,13 @@ __global__ void __launch_bounds__(1024) tile_order_kernel(const uint32_t *ranges
 // one kernel of one CTA, the pairs held in shared memory between the passes.
 // The general path is 10 kernels and two memsets whatever the count: with the
 // one-kernel intersect this takes a preview frame of about a thousand pairs
-// from 119 to 49 us. Above 8192 pairs the one SM would hold the frame up
-// longer than the launches.
+// from 119 to 49 us. The lines, by the time of the sort alone with all pairs
+// in use (one CTA / general, in us): 1000 pairs, 300 tiles 24 / 82 launched one
+// by one and 22 / 60 in a graph; 8192 pairs, 300 tiles 70 / 87 and 67 / 69.
+// Beyond, the one SM would hold a replayed frame up longer than ten small
+// launches. It also walks the tiles alone (1 us per 1024): 8192 pairs, 16384
+// tiles 88 / 104, but 86 / 78 in a graph. Ending at fewer pairs there was not
+// kept: a 1419x1080 frame of 5.6k pairs, launched plainly, went from 235 to 282 us.
 constexpr int kSmallThreads = 1024;
 constexpr int kSmallWarps = kSmallThreads / 32;
 constexpr int kSmallItems = 8;

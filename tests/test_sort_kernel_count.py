@@ -21,6 +21,9 @@ def test_counts(lib):
     assert psi.sort_kernel_count(1 << 20, 0, 45, 0) == 2 + 6
     assert psi.sort_kernel_count(1 << 20, 0, 33, 300) == 2 + 6 + 2    # 5 digits: an even number of passes
     assert psi.sort_kernel_count(1 << 20, 0, 64, 300) == 2 + 8 + 2
+    # the one-CTA form: up to 8192 pairs and, with ranges, 16384 tiles
+    for cap, tiles, one in ((8192, 16384, True), (8193, 16384, False), (8192, 16385, False), (8192, 0, True)):
+        assert (psi.sort_kernel_count(cap, 0, 45, tiles) == 1) == one, (cap, tiles)
     k = ctypes.c_int(0)
     for bad in ((-1, 0, 45, 1), (10, -1, 45, 1), (10, 0, 65, 1), (10, 5, 5, 1), (10, 0, 45, -1)):
         assert lib.psi_sort_kernel_count(*bad, ctypes.byref(k)) == psi.PSI_ERR_INVALID_ARG
